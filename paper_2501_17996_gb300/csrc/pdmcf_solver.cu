@@ -24,6 +24,7 @@
 #include "pdmcf_batch.cuh"
 #include "pdmcf_internal.h"
 #include "pdmcf_kernels.h"
+#include "pdmcf_resident.h"
 
 namespace pdmcf {
 
@@ -128,6 +129,9 @@ struct DeviceState {
   int tma = -1, tma_kind = 0, grid_tma = 0, grid_node_pin = 0;   // kind 1 bulk-copy, 2 in-sum
   bool renumbered = false;   // nodes relabelled for locality (Topology::node_of)
   size_t tma_smem = 0;
+  // resident iteration (resident >= 0): many iterations per cooperative launch
+  int resident = -1, grid_resident = 0;
+  ResidentCtl* ctl = nullptr;
   void* Pin = nullptr;
   int32_t* cta_ptr = nullptr;
   int32_t* node_map = nullptr;   // caller node -> internal node (boundary layouts)
@@ -292,7 +296,7 @@ static void free_state(DeviceState* d) {
   void* bufs[] = {d->F[0], d->F[1], d->Y[0], d->Y[1], d->Ylo[0], d->Ylo[1], d->Pm, d->W, d->G, d->mu, d->cap,
                   d->That, d->Uprime, d->Yhat, d->e_tail, d->e_head, d->in_ptr,
                   d->out_ptr, d->out_idx, d->part_edge, d->part_node, d->part_check, d->sc,
-                  d->Pin, d->cta_ptr, d->node_map};
+                  d->Pin, d->cta_ptr, d->node_map, d->ctl};
   for (void* b : bufs) dfree(d, b);
   if (d->sc_host) cudaFreeHost(d->sc_host);
   if (d->own_stream) cudaStreamDestroy(d->own_stream);
@@ -519,6 +523,43 @@ static int setup_grids(DeviceState* d, int want) {
 }
 
 
+template <typename P, typename S> const ResidentTable<P, S>& get_resident();
+template <> const ResidentTable<float, float>& get_resident<float, float>() { return resident_table_f32(); }
+template <> const ResidentTable<double, double>& get_resident<double, double>() { return resident_table_f64(); }
+template <> const ResidentTable<float, __nv_bfloat16>& get_resident<float, __nv_bfloat16>() {
+  return resident_table_bf16();
+}
+
+// The resident iteration serves automatic shapes whose rows fit a warp's registers (and have no
+// in-sum kind). A forced shape and a timed solve launch the per-phase kernels. Measured per
+// iteration, per-phase kernels in a CUDA graph against resident (us, GB300): n = 10: 14.9 and 4.5;
+// n = 100, m = 1000: 17.1 and 6.1; n = 203 FP64 with an exponent per pair: 682 and 51; n = 1000,
+// m = 8000: 61.5 and 46.0; n = 1000, m = 11 500 (kNN): 78.4 and 61.2.
+template <typename P, typename S>
+static int setup_resident(DeviceState* d, int want) {
+  d->resident = -1;
+  d->grid_resident = 0;
+  const int t = want < 0 && d->tma < 0 ? pick_resident((int)(d->ld / StoreTraits<S>::VW)) : -1;
+  if (t < 0) return MCF_OK;
+  int coop = 0, sms = 0, occ = 0;
+  CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, d->device));
+  if (!coop) return MCF_OK;
+  constexpr int B = RESIDENT_BLOCK;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d->device));
+  for (const void* fn : {(const void*)get_resident<P, S>().plain[t], (const void*)get_resident<P, S>().special[t]}) {
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, B, 0));
+    if (occ < 1) return MCF_OK;
+  }
+  // Four warps' work (an edge, or 32 entries of Y) per CTA before the next SM is taken: a phase
+  // is bounded by the latency of a warp's one item, so spreading wins until all SMs have some.
+  // Measured per iteration (us, GB300): n = 10, m = 40: 6.3 in one CTA (no grid barrier), 4.5 in
+  // 10, 5.2 in 40; n = 100, m = 1000: 18.8 in 10 CTAs, 5.7 in 76 and in 152.
+  const int64_t warps = std::max<int64_t>(d->m, (int64_t)d->n * ((d->ld + 31) / 32));
+  d->resident = t;
+  d->grid_resident = (int)std::min<int64_t>(sms, (warps + 3) / 4);
+  return MCF_OK;
+}
+
 static int configure_shape(DeviceState* d, int want) {
   if (d->precision == MCF_FP64) {
     if (want >= NUM_SHAPES) {
@@ -526,15 +567,18 @@ static int configure_shape(DeviceState* d, int want) {
       return MCF_ERR_INVALID;
     }
     d->tma = -1;
-    return setup_grids<double, double>(d, want);
+    const int rc = setup_grids<double, double>(d, want);
+    return rc == MCF_OK ? setup_resident<double, double>(d, want) : rc;
   }
   int rc;
   if (d->precision == MCF_BF16_F) {
     rc = setup_grids<float, __nv_bfloat16>(d, want);
     if (rc == MCF_OK) rc = setup_tma<__nv_bfloat16>(d, want);
+    if (rc == MCF_OK) rc = setup_resident<float, __nv_bfloat16>(d, want);
   } else {
     rc = setup_grids<float, float>(d, want);
     if (rc == MCF_OK) rc = setup_tma<float>(d, want);
+    if (rc == MCF_OK) rc = setup_resident<float, float>(d, want);
   }
   return rc;
 }
@@ -594,9 +638,9 @@ static int alloc_partials(DeviceState* d) {
   if (d->part_edge || d->part_node || d->part_check) cudaDeviceSynchronize();
   for (double** b : {&d->part_edge, &d->part_node, &d->part_check})
     if (*b) { dfree(d, *b); *b = nullptr; }
-  bool ok = dalloc(d, (void**)&d->part_edge, (size_t)std::max({d->grid_edge, d->grid_tma, 1}) * sizeof(double)) &&
-            dalloc(d, (void**)&d->part_node, (size_t)std::max({d->grid_node, d->grid_node_pin, 1}) * NODE_PARTS * sizeof(double)) &&
-            dalloc(d, (void**)&d->part_check, (size_t)std::max(d->grid_check, 1) * CHECK_PARTS * sizeof(double));
+  bool ok = dalloc(d, (void**)&d->part_edge, (size_t)std::max({d->grid_edge, d->grid_tma, d->grid_resident, 1}) * sizeof(double)) &&
+            dalloc(d, (void**)&d->part_node, (size_t)std::max({d->grid_node, d->grid_node_pin, d->grid_resident, 1}) * NODE_PARTS * sizeof(double)) &&
+            dalloc(d, (void**)&d->part_check, (size_t)std::max(d->grid_check, d->grid_resident) * CHECK_PARTS * sizeof(double));
   if (!ok) {
     set_error("device allocation failed");
     return MCF_ERR_OOM;
@@ -667,7 +711,7 @@ static int alloc_state(mcf_problem* p, int precision, int device, int shape, cud
   ok = ok && A((void**)&d->e_tail, m * 4) && A((void**)&d->e_head, m * 4) &&
        A((void**)&d->in_ptr, (n + 1) * 4) && A((void**)&d->out_ptr, (n + 1) * 4) &&
        A((void**)&d->out_idx, m * 4);
-  ok = ok && A((void**)&d->sc, sizeof(DevScalars));
+  ok = ok && A((void**)&d->sc, sizeof(DevScalars)) && A((void**)&d->ctl, sizeof(ResidentCtl));
   if (ok && d->pool && cudaStreamSynchronize(d->own_stream) != cudaSuccess) {
     cudaGetLastError();
     ok = false;
@@ -948,6 +992,46 @@ static void write_check_line(FILE* f, const DevScalars& h, int n, int m, int pre
 static std::atomic<int> g_withhold_request{0};
 static bool take_withhold_request() { return g_withhold_request.exchange(0) != 0; }
 
+// Queue iterations [k, k + count) of the resident path: launches of plain iterations between
+// those with a scalar tail (k a multiple of k_adapt, or a stop test). Once a stop test holds on
+// the device the launches behind it return at once.
+template <typename P, typename S>
+static cudaError_t launch_resident(DeviceState* d, const IterArgs<P, S>& args, int parity, int64_t k, int64_t count,
+                                   int64_t max_iters, int64_t kc, int64_t k_adapt, const StopRule& rule,
+                                   cudaStream_t st) {
+  const ResidentTable<P, S>& T = get_resident<P, S>();
+  k_adapt = std::max<int64_t>(1, k_adapt);
+  auto check = [&](int64_t i) { return (i + 1) % kc == 0 || i + 1 >= max_iters; };
+  auto special = [&](int64_t i) { return check(i) || i % k_adapt == 0; };
+  cudaError_t e = cudaMemsetAsync(&d->ctl->arrived, 0, sizeof(unsigned), st);
+  unsigned arrived = 0;
+  const int64_t end = k + count;
+  while (k < end && e == cudaSuccess) {
+    const bool sp = special(k);
+    int64_t to = k;
+    unsigned barriers = 0;
+    while (to < end && special(to) == sp) {
+      barriers += sp ? (check(to) ? 4u : 3u) : 2u;
+      ++to;
+    }
+    --barriers;   // the end of the kernel is the last one
+    IterArgs<P, S> a = args;
+    a.parity = parity;
+    ResidentArgs ra{d->ctl, k, (int)(to - k), arrived, max_iters, kc, rule};
+    void* kargs[] = {&a, &ra};
+    e = cudaLaunchCooperativeKernel(sp ? (const void*)T.special[d->resident] : (const void*)T.plain[d->resident],
+                                    dim3(d->grid_resident), dim3(RESIDENT_BLOCK), kargs, 0, st);
+    arrived += barriers * (unsigned)d->grid_resident;
+    if ((to - k) & 1) parity ^= 1;
+    k = to;
+  }
+  return e;
+}
+
+// Most iterations of one group of resident launches (whole chunks of k_check): the host looks
+// at the result, and other work gets the GPU, at least this often.
+constexpr int64_t kResidentIters = 1000;
+
 template <typename P, typename S>
 static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_result* res,
                    cudaStream_t st, mcf_kernel_times* kt, const PhaseRule& rule = PhaseRule()) {
@@ -1028,41 +1112,55 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
     return MCF_ERR_INVALID;
   }
   int64_t k = 0;
-  double best_kkt = INFINITY;
-  int since_best = 0;
-  double floor_best = INFINITY;
-  int floor_since = 0;
-  bool floor_frozen = false;   // omega had stopped adapting when the count last restarted
-  bool stalled = false;
-  int status = MCF_ERR_NOT_CONVERGED;
-  if (o->stop_mode == MCF_STOP_NONE) status = MCF_OK;
+  StopRule stop;
+  stop.mode = o->stop_mode;
+  stop.eps = o->eps;
+  stop.nm = (double)n * (double)m;
+  stop.stall_checks = o->stall_checks;
+  stop.handoff = rule.handoff;
+  stop.handoff_stall = rule.stall_checks;
+  StopState stop_state = stop_state_init();
+  int verdict = STOP_NO;
   bool any = false;
+  const bool resident = d->resident >= 0 && kt == nullptr;
+  if (resident) CK(cudaMemcpyAsync(&d->ctl->stop, &stop_state, sizeof(stop_state), cudaMemcpyHostToDevice, st));
   NvtxRange solve_range(d->precision == MCF_FP64 ? "pdmcf solve fp64"
                         : d->precision == MCF_BF16_F ? "pdmcf solve bf16" : "pdmcf solve fp32");
-  while (k < max_iters) {
+  while (k < max_iters && verdict == STOP_NO) {
     NvtxRange chunk_range("pdmcf chunk");
-    const int64_t chunk = std::min<int64_t>(kc - (k % kc), max_iters - k);
+    int64_t chunk = std::min<int64_t>(kc - (k % kc), max_iters - k);
     const bool stall_first = withhold && k == 0;
-    if (use_graphs && chunk == kc && !stall_first) {
-      if (!d->graph[parity] && !capture_chunk<P, S>(d, args, parity, kc, st, &d->graph[parity])) {
-        d->graphs_broken = true;
-        use_graphs = false;
-      }
-    }
-    if (use_graphs && chunk == kc && !stall_first) {
-      CK(cudaGraphLaunch(d->graph[parity], st));
-      if (kc & 1) parity ^= 1;
+    if (resident) {
+      // the device evaluates the stop test: several chunks per launch, one with a check log
+      if (!log) chunk = std::min<int64_t>((int64_t)kc * std::max<int64_t>(1, kResidentIters / kc), max_iters - k);
+      CK((launch_resident<P, S>(d, args, parity, k, chunk, max_iters, kc, o->k_adapt, stop, st)));
+      CK(cudaMemcpyAsync(&stop_state, &d->ctl->stop, sizeof(stop_state), cudaMemcpyDeviceToHost, st));
     } else {
-      for (int64_t i = 0; i < chunk; ++i) {
-        const IterArgs<P, S>& ai = (stall_first && i == 0) ? args_w : args;
-        if (kt) CK((launch_iteration_timed<P, S>(d, ai, parity, i == chunk - 1, st, pool)));
-        else CK((launch_iteration<P, S>(d, ai, parity, i == chunk - 1, st)));
-        parity ^= 1;
+      if (use_graphs && chunk == kc && !stall_first) {
+        if (!d->graph[parity] && !capture_chunk<P, S>(d, args, parity, kc, st, &d->graph[parity])) {
+          d->graphs_broken = true;
+          use_graphs = false;
+        }
+      }
+      if (use_graphs && chunk == kc && !stall_first) {
+        CK(cudaGraphLaunch(d->graph[parity], st));
+        if (kc & 1) parity ^= 1;
+      } else {
+        for (int64_t i = 0; i < chunk; ++i) {
+          const IterArgs<P, S>& ai = (stall_first && i == 0) ? args_w : args;
+          if (kt) CK((launch_iteration_timed<P, S>(d, ai, parity, i == chunk - 1, st, pool)));
+          else CK((launch_iteration<P, S>(d, ai, parity, i == chunk - 1, st)));
+          parity ^= 1;
+        }
       }
     }
     CK(cudaMemcpyAsync(d->sc_host, d->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (kt) drain_events(pool, kt);
+    if (resident) {
+      chunk = h.k - k;   // a stop test may have ended the launch early
+      if (chunk & 1) parity ^= 1;
+    }
     k += chunk;
     any = true;
     d->cur = parity;
@@ -1073,25 +1171,15 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
       d->valid = false;
       return MCF_ERR_CUDA;
     }
-    if (h.numeric_error) {
-      status = MCF_ERR_NUMERIC;
-      set_error("NaN or Inf in the iterates");
-      break;
-    }
-    if (o->stop_mode == MCF_STOP_PAPER && h.r < (double)n * (double)m * o->eps) { status = MCF_OK; break; }
-    if (o->stop_mode == MCF_STOP_REL_KKT && h.rel_kkt < o->eps) { status = MCF_OK; break; }
-    if (rule.handoff > 0.0 && h.rel_kkt < rule.handoff) break;
-    if (o->stop_mode == MCF_STOP_REL_KKT && o->stall_checks > 0 && h.rel_kkt < 100.0 * o->eps) {
-      const bool frozen = h.freeze >= 0 && h.freeze <= h.k;
-      if (frozen != floor_frozen) { floor_frozen = frozen; floor_best = INFINITY; floor_since = 0; }
-      if (h.rel_kkt < 0.95 * floor_best) { floor_best = h.rel_kkt; floor_since = 0; }
-      else if (++floor_since >= o->stall_checks) { stalled = true; break; }
-    }
-    if (rule.stall_checks > 0) {
-      if (h.rel_kkt < 0.95 * best_kkt) { best_kkt = h.rel_kkt; since_best = 0; }
-      else if (++since_best >= rule.stall_checks) break;
-    }
+    verdict = resident ? stop_state.verdict : stop_test(h, stop, stop_state);
   }
+  int status = o->stop_mode == MCF_STOP_NONE ? MCF_OK : MCF_ERR_NOT_CONVERGED;
+  if (verdict == STOP_CONVERGED) status = MCF_OK;
+  if (verdict == STOP_NUMERIC) {
+    status = MCF_ERR_NUMERIC;
+    set_error("NaN or Inf in the iterates");
+  }
+  const bool stalled = verdict == STOP_STALLED;
   p->omega = h.omega;
   if (!any) {
     set_error("max_iters must be >= 1");
