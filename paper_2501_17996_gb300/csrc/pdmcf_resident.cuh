@@ -184,19 +184,16 @@ __device__ __forceinline__ int node_edge(const IterArgs<P, S>& a, const NodePiec
   return l < q.nin ? q.ib + l : __ldg(a.out_idx + q.ob + l - q.nin);
 }
 
+// Piece `p` of the n x per pieces, node index fastest; the edges are loaded by node_edge.
 template <typename P, typename S, int N>
-__device__ __forceinline__ void node_place(const IterArgs<P, S>& a, unsigned piece, unsigned per, NodePiece& q) {
-  const int lane = threadIdx.x & 31;
-  const int j = (int)(piece / per);
-  q.c = (int)(piece - (unsigned)j * per) * 32 + lane;
-  if (j != q.j) {
-    q.j = j;
-    q.ib = __ldg(a.in_ptr + j);
-    q.nin = __ldg(a.in_ptr + j + 1) - q.ib;
-    q.ob = __ldg(a.out_ptr + j);
-    q.deg = q.nin + __ldg(a.out_ptr + j + 1) - q.ob;
-    q.edge = node_edge(a, q, lane);
-  }
+__device__ __forceinline__ void node_place(const IterArgs<P, S>& a, unsigned p, NodePiece& q) {
+  const unsigned c = p / (unsigned)a.n;
+  q.j = (int)(p - c * (unsigned)a.n);
+  q.c = (int)c * 32 + (int)(threadIdx.x & 31);
+  q.ib = __ldg(a.in_ptr + q.j);
+  q.nin = __ldg(a.in_ptr + q.j + 1) - q.ib;
+  q.ob = __ldg(a.out_ptr + q.j);
+  q.deg = q.nin + __ldg(a.out_ptr + q.j + 1) - q.ob;
 }
 
 // What does not depend on the edge phase: data (constant) and state of a piece.
@@ -216,7 +213,7 @@ __device__ __forceinline__ void node_data(const IterArgs<P, S>& a, const NodePie
 #pragma unroll
     for (int u = 0; u < N; ++u) x.gv[u] = a.gamma;
   }
-  if (a.kind == 1) {
+  if (a.kind == 1 && sizeof(S) != 2) {
 #pragma unroll
     for (int u = 0; u < N; ++u)
       x.wg[u] = x.gv[u] == P(0.5) ? P(0) : pow(x.wv[u] * x.gv[u], P(1) / (P(1) - x.gv[u]));
@@ -248,10 +245,11 @@ __device__ __forceinline__ void node_rows(const S* __restrict__ f0, size_t ld, i
   for (int r = 0; r < R; ++r)
     ld_words<S, N>(f0 + (size_t)__shfl_sync(0xffffffffu, edge, k + r) * ld, f[r]);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const P sg = k + r < nin ? P(1) : k + r < deg ? P(-1) : P(0);
+  for (int r = 0; r < R; r += 2) {   // consecutive pairs, as node_kernel adds them
+    const P s0 = k + r < nin ? P(1) : k + r < deg ? P(-1) : P(0);
+    const P s1 = k + r + 1 < nin ? P(1) : k + r + 1 < deg ? P(-1) : P(0);
 #pragma unroll
-    for (int u = 0; u < N; ++u) s[u] = fma(sg, to_p<P>(f[r][u]), s[u]);
+    for (int u = 0; u < N; ++u) s[u] += fma(s0, to_p<P>(f[r][u]), s1 * to_p<P>(f[r + 1][u]));
   }
 }
 
@@ -271,9 +269,13 @@ __device__ __forceinline__ void node_gather(const IterArgs<P, S>& a, const S* __
     if (N == 1 && cnt > 16) {
       node_rows<P, S, N, 24>(f0, a.ld, edge, 0, nin, deg, s);
       k = 24;
-    } else if (cnt > 12) {
+    } else if (N <= 2 && cnt > 12) {
       node_rows<P, S, N, 16>(f0, a.ld, edge, 0, nin, deg, s);
       k = 16;
+    }
+    if constexpr (N > 2) {
+#pragma unroll 1
+      for (; k + 6 < cnt; k += 8) node_rows<P, S, N, 8>(f0, a.ld, edge, k, nin, deg, s);
     }
 #pragma unroll 1
     for (; k < cnt; k += 4) node_rows<P, S, N, 4>(f0, a.ld, edge, k, nin, deg, s);
@@ -298,7 +300,9 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
     P delta, tr = P(0);
     if (live) {
       const P vv = x.yo[u] + (x.yl[u] - beta * fplus_at);
-      if (a.kind == 0) tr = prox_traffic<P>(0, vv, beta, x.wv[u], x.gv[u]);
+      // (with BF16-stored F a last-place difference of Y flips roundings of F, so that path
+      // keeps the search of node_kernel, to the bit)
+      if (a.kind == 0 || sizeof(S) == 2) tr = prox_traffic<P>(a.kind, vv, beta, x.wv[u], x.gv[u]);
       else prox_pow_traffic<P>(vv, beta, x.wv[u], x.wg[u], x.gv[u], tr);
       delta = -beta * (fplus_at + tr);
     } else {
@@ -345,26 +349,32 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
   }
 }
 
-// Pieces [p0, p1) of the node phase, consecutive ones of the n columns: every warp of the grid
-// has about as many (a warp per node left 5 of 6 SMs idle at n = 200), a thread's serial chain
-// is N root searches instead of a whole row's, and the next piece's data is loaded while this
-// one's rows arrive.
+// The node phase. Every warp of the grid has about as many pieces (a warp per node left 5 of 6
+// SMs idle at n = 200), and a thread's serial chain is N root searches instead of a whole row's.
+// Pieces go column block by column block over all nodes, so that the rows of a block that nodes
+// gather (each row by its head and by its tail) are in L2 together: F is read from HBM once
+// where it does not fit L2. The next piece's edges and data are loaded while this one's rows
+// arrive.
 template <typename P, typename S, int N, bool CHECK>
 __device__ __forceinline__ void node_pieces(const IterArgs<P, S>& a, int par, unsigned p0, unsigned p1,
-                                            unsigned per, NodePiece& q, NodeItem<P, N>& x, P beta,
+                                            unsigned step, NodePiece& q, NodeItem<P, N>& x, P beta,
                                             double (&acc)[NODE_PARTS]) {
   const S* Fn = a.F[par ^ 1];
 #pragma unroll 1
-  for (unsigned pc = p0; pc < p1; ++pc) {
+  for (unsigned pc = p0; pc < p1; pc += step) {
     P s[N], loc[NODE_PARTS];
 #pragma unroll
     for (int k = 0; k < NODE_PARTS; ++k) loc[k] = P(0);
+    const bool more = pc + step < p1;
+    NodePiece qn;
+    if (more) node_place<P, S, N>(a, pc + step, qn);
     node_gather<P, S, N>(a, Fn, q, s);
+    if (more) qn.edge = node_edge(a, qn, (int)(threadIdx.x & 31));
     node_update<P, S, N, CHECK>(a, par, q, s, x, beta, loc);
 #pragma unroll
     for (int k = 0; k < (CHECK ? NODE_PARTS : 1); ++k) acc[k] += (double)loc[k];
-    if (pc + 1 < p1) {
-      node_place<P, S, N>(a, pc + 1, per, q);
+    if (more) {
+      q = qn;
       node_data<P, S, N>(a, q, x);
       node_state<P, S, N>(a, par, q, x);
     }
@@ -432,7 +442,7 @@ __device__ __forceinline__ void check_phase(const IterArgs<P, S>& a, int par, P 
   }
 }
 
-// ------------------------------------------------------------------ the kernel
+// ------------------------------------------------------------------ scalar tail
 
 // Scalar tail in block 0: a warp per field sums the CTAs' FP64 partials in a fixed order, then
 // one thread updates the scalars and evaluates the stop test.
@@ -665,26 +675,23 @@ __device__ __forceinline__ P edge_phase(const IterArgs<P, S>& a, int par, P alph
   return dsum;
 }
 
-// ------------------------------------------------------------------ the kernel
+// ------------------------------------------------------------------ the kernels
 
 struct ResidentPlace {   // this warp's share of the work
   int e0, e1, warp, nwarps;
-  unsigned p0, p1, per;
+  unsigned pieces;   // of the node phase: this warp takes warp, warp + nwarps, ...
 };
 
 template <int NW>
 __device__ __forceinline__ ResidentPlace resident_place(int n, int m, int ld, int N) {
   ResidentPlace w;
-  w.warp = blockIdx.x * NW + (threadIdx.x >> 5);
+  // numbered across the CTAs first, so that few pieces spread over all SMs
+  w.warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   w.nwarps = gridDim.x * NW;
-  // consecutive edges per CTA (their heads' dual rows are shared in L1), consecutive pieces of
-  // the node phase per warp
+  // consecutive edges per CTA (their heads' dual rows are shared in L1)
   w.e0 = (int)((long long)m * blockIdx.x / gridDim.x) + (threadIdx.x >> 5);
   w.e1 = (int)((long long)m * (blockIdx.x + 1) / gridDim.x);
-  w.per = (unsigned)(ld + 32 * N - 1) / (32 * N);
-  const unsigned long long total = (unsigned long long)n * w.per;
-  w.p0 = (unsigned)(total * w.warp / w.nwarps);
-  w.p1 = (unsigned)(total * (w.warp + 1) / w.nwarps);
+  w.pieces = (unsigned)n * ((unsigned)(ld + 32 * N - 1) / (32 * N));
   return w;
 }
 
@@ -700,8 +707,10 @@ resident_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant_
   const P alpha = (P)__ldcg(&a.sc->alpha), beta = (P)__ldcg(&a.sc->beta);
   NodePiece piece;
   NodeItem<P, N> x;      // data of the first piece: stays in registers when it is the only one
-  if (w.p0 < w.p1) {
-    node_place<P, S, N>(a, w.p0, w.per, piece);
+  const bool any = (unsigned)w.warp < w.pieces, one = (unsigned)(w.warp + w.nwarps) >= w.pieces;
+  if (any) {
+    node_place<P, S, N>(a, w.warp, piece);
+    piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
     node_data<P, S, N>(a, piece, x);
   }
   if (threadIdx.x == 0) failed = 0;
@@ -714,16 +723,17 @@ resident_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant_
     const P dsum = edge_phase<P, S, VPT, NW>(a, par, alpha, w.e0, w.e1, bar, i > 0, ok);
     if (!ok) return;
     bar.arrive();
-    if (w.p0 < w.p1) {
-      if (w.p0 + 1 < w.p1) {
-        node_place<P, S, N>(a, w.p0, w.per, piece);
+    if (any) {
+      if (!one) {
+        node_place<P, S, N>(a, w.warp, piece);
+        piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
         node_data<P, S, N>(a, piece, x);
       }
       node_state<P, S, N>(a, par, piece, x);
     }
     if (!bar.wait()) return;
     double acc[NODE_PARTS] = {0.0};
-    node_pieces<P, S, N, false>(a, par, w.p0, w.p1, w.per, piece, x, beta, acc);
+    node_pieces<P, S, N, false>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
     // a sum that is not finite here is reported as the scalar tail would
     if (!isfinite(dsum) || !isfinite(acc[0])) a.sc->numeric_error = 1;
     if (i + 1 < ra.count) bar.arrive();
@@ -756,13 +766,14 @@ resident_special_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_c
     for (int q = 0; q < NODE_PARTS; ++q) acc[q] = 0.0;
     NodePiece piece;
     NodeItem<P, N> x;
-    if (w.p0 < w.p1) {
-      node_place<P, S, N>(a, w.p0, w.per, piece);
+    if ((unsigned)w.warp < w.pieces) {
+      node_place<P, S, N>(a, w.warp, piece);
+      piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
       node_data<P, S, N>(a, piece, x);
       node_state<P, S, N>(a, par, piece, x);
     }
-    if (check) node_pieces<P, S, N, true>(a, par, w.p0, w.p1, w.per, piece, x, beta, acc);
-    else node_pieces<P, S, N, false>(a, par, w.p0, w.p1, w.per, piece, x, beta, acc);
+    if (check) node_pieces<P, S, N, true>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
+    else node_pieces<P, S, N, false>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
     double v1[1] = {(double)dsum};
     block_sum_write<BLOCK, 1>(v1, a.part_edge + blockIdx.x);
     block_sum_write<BLOCK, NODE_PARTS>(acc, a.part_node + (size_t)blockIdx.x * NODE_PARTS);
@@ -783,14 +794,13 @@ resident_special_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_c
   }
 }
 
-// Entries per lane of a piece: one where a row has at most 512 entries (few pieces per warp),
-// else two.
 template <typename P, typename S, int IDX>
 void fill_resident(ResidentTable<P, S>& t) {
-  constexpr int V = kResidentVpt[IDX];
-  constexpr int N = 32 * StoreTraits<S>::VW * V <= 512 ? 1 : 2;
-  t.plain[IDX] = resident_kernel<P, S, V, N, RESIDENT_BLOCK>;
-  t.special[IDX] = resident_special_kernel<P, S, V, N, RESIDENT_BLOCK>;
+  constexpr ResidentVariant v = resident_variant<P, S>(IDX);
+  if constexpr (32 * v.vpt * StoreTraits<S>::VW <= 1024) {
+    t.plain[IDX] = resident_kernel<P, S, v.vpt, v.entries, RESIDENT_BLOCK>;
+    t.special[IDX] = resident_special_kernel<P, S, v.vpt, v.entries, RESIDENT_BLOCK>;
+  }
 }
 template <typename P, typename S>
 ResidentTable<P, S> make_resident_table() {

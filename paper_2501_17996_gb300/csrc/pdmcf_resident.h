@@ -67,10 +67,18 @@ struct ResidentArgs {
   StopRule rule;
 };
 
-// A warp owns an edge (VPT chunks per lane), a thread a few entries of a node's column.
+// Variants by row length: a warp owns an edge (`vpt` chunks per lane), a lane `entries` of a piece of
+// a node's column; one CTA of 512 threads per SM (128 registers each). Rows longer than eight
+// chunks per lane were tried with 384 threads and stay with the per-phase kernels: at n = 3000
+// an iteration took 607 us against 367 (twelve warps per SM do not cover the node phase's loads).
+struct ResidentVariant { int vpt, entries; };
+constexpr int RESIDENT_BLOCK = 512;
 constexpr int NUM_RESIDENT = 4;
-constexpr int kResidentVpt[NUM_RESIDENT] = {1, 2, 4, 8};
-constexpr int RESIDENT_BLOCK = 512;   // one CTA per SM, 128 registers per thread
+template <typename P, typename S>
+constexpr ResidentVariant resident_variant(int i) {
+  constexpr int vpt[NUM_RESIDENT] = {1, 2, 4, 8};
+  return {vpt[i], 32 * StoreTraits<S>::VW * vpt[i] <= 512 ? 1 : 2};
+}
 
 // `plain` runs iterations without a scalar tail, `special` those with one (a multiple of k_adapt,
 // or a stop test).
@@ -81,12 +89,13 @@ struct ResidentTable {
 };
 const ResidentTable<float, float>& resident_table_f32();
 const ResidentTable<double, double>& resident_table_f64();
-const ResidentTable<float, __nv_bfloat16>& resident_table_bf16();
+const ResidentTable<float, __nv_bfloat16>& resident_table_bf16();   // three variants: rows of 1024 entries
 
 // Index of the smallest variant that covers nchunks chunks per row, -1 if none does.
+template <typename P, typename S>
 inline int pick_resident(int nchunks) {
   for (int t = 0; t < NUM_RESIDENT; ++t)
-    if (32 * kResidentVpt[t] >= nchunks) return t;
+    if (32 * resident_variant<P, S>(t).vpt >= nchunks) return t;
   return -1;
 }
 

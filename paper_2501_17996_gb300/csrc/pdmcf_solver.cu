@@ -24,6 +24,7 @@
 #include "pdmcf_batch.cuh"
 #include "pdmcf_internal.h"
 #include "pdmcf_kernels.h"
+#include "pdmcf_flat.h"
 #include "pdmcf_resident.h"
 
 namespace pdmcf {
@@ -48,6 +49,7 @@ struct ScalarArgs {
   const double* pc;
   int nbc;
   int check;
+  long long k;        // iterations completed before this one (-1: as counted by the scalars)
 };
 
 __global__ void __launch_bounds__(256) scalar_kernel(ScalarArgs a) {
@@ -61,6 +63,7 @@ __global__ void __launch_bounds__(256) scalar_kernel(ScalarArgs a) {
     for (int f = 0; f < CHECK_PARTS; ++f) chk[f] = det_sum(a.pc, a.nbc, CHECK_PARTS, f, sh);
   }
   if (threadIdx.x != 0) return;
+  if (a.k >= 0) a.sc->k = a.k;
   scalar_update(a.sc, dF2, dY2, nodep, chk, a.check != 0);
 }
 
@@ -127,11 +130,15 @@ struct DeviceState {
   int requested_shape = -1;   // mcf_options.shape the grids were configured for
   // pipelined edge phase (tma >= 0): one CTA per SM over head-aligned edge ranges
   int tma = -1, tma_kind = 0, grid_tma = 0, grid_node_pin = 0;   // kind 1 bulk-copy, 2 in-sum
+  bool general_pow = false;  // power utility with an exponent other than 1/2
   bool renumbered = false;   // nodes relabelled for locality (Topology::node_of)
   size_t tma_smem = 0;
   // resident iteration (resident >= 0): many iterations per cooperative launch
   int resident = -1, grid_resident = 0;
   ResidentCtl* ctl = nullptr;
+  // iterations without a scalar tail where the resident iteration does not serve: the register
+  // edge phase and the node phase over pieces (grid_flat > 0)
+  int grid_flat = 0;
   void* Pin = nullptr;
   int32_t* cta_ptr = nullptr;
   int32_t* node_map = nullptr;   // caller node -> internal node (boundary layouts)
@@ -539,8 +546,8 @@ template <typename P, typename S>
 static int setup_resident(DeviceState* d, int want) {
   d->resident = -1;
   d->grid_resident = 0;
-  const int t = want < 0 && d->tma < 0 ? pick_resident((int)(d->ld / StoreTraits<S>::VW)) : -1;
-  if (t < 0) return MCF_OK;
+  const int t = want < 0 && d->tma < 0 ? pick_resident<P, S>((int)(d->ld / StoreTraits<S>::VW)) : -1;
+  if (t < 0 || d->ld > 1024) return MCF_OK;   // (BF16, n = 2000: 151 us per-phase, 175 us resident)
   int coop = 0, sms = 0, occ = 0;
   CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, d->device));
   if (!coop) return MCF_OK;
@@ -560,6 +567,32 @@ static int setup_resident(DeviceState* d, int want) {
   return MCF_OK;
 }
 
+template <typename P, typename S> const void* flat_kernel();
+template <> const void* flat_kernel<float, float>() { return (const void*)flat_kernel_f32(); }
+template <> const void* flat_kernel<float, __nv_bfloat16>() { return (const void*)flat_kernel_bf16(); }
+template <> const void* flat_kernel<double, double>() { return (const void*)flat_kernel_f64(); }
+
+// Iterations without a scalar tail on automatic shapes that are not resident: the register edge
+// phase and the flat node phase, against the kernels of setup_grids / setup_tma (us per iteration,
+// GB300, out-degree 8 log or 10 power). FP64: n = 700 393 -> 364, with an exponent per pair
+// 1314 -> 638. Networks without node locality: n = 1500 87 -> 83, n = 2500 299 -> 221 (FP32) and
+// 276 -> 188 (BF16), n = 3500 459 -> 427, n = 4000 power 661 -> 689 (the in-sum kind stays).
+// Renumbered networks, where the node phase's rows are close in memory anyway: n = 1500 113 -> 111,
+// n = 2000 178 -> 184. With exponents other than 1/2 the flat phase's root search decides:
+// n = 3000 559 -> 426.
+template <typename P, typename S>
+static int setup_flat(DeviceState* d, int want) {
+  d->grid_flat = 0;
+  if (want >= 0 || d->resident >= 0) return MCF_OK;
+  const int most = sizeof(P) == 8 ? INT32_MAX : d->general_pow ? 4096 : d->renumbered ? 1536 : 3584;
+  if (d->ld > most) return MCF_OK;
+  int sms = 0, occ = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d->device));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (flat_kernel<P, S>()), FLAT_BLOCK, 0));
+  d->grid_flat = std::max(1, occ) * sms;
+  return MCF_OK;
+}
+
 static int configure_shape(DeviceState* d, int want) {
   if (d->precision == MCF_FP64) {
     if (want >= NUM_SHAPES) {
@@ -567,18 +600,21 @@ static int configure_shape(DeviceState* d, int want) {
       return MCF_ERR_INVALID;
     }
     d->tma = -1;
-    const int rc = setup_grids<double, double>(d, want);
-    return rc == MCF_OK ? setup_resident<double, double>(d, want) : rc;
+    int rc = setup_grids<double, double>(d, want);
+    if (rc == MCF_OK) rc = setup_resident<double, double>(d, want);
+    return rc == MCF_OK ? setup_flat<double, double>(d, want) : rc;
   }
   int rc;
   if (d->precision == MCF_BF16_F) {
     rc = setup_grids<float, __nv_bfloat16>(d, want);
     if (rc == MCF_OK) rc = setup_tma<__nv_bfloat16>(d, want);
     if (rc == MCF_OK) rc = setup_resident<float, __nv_bfloat16>(d, want);
+    if (rc == MCF_OK) rc = setup_flat<float, __nv_bfloat16>(d, want);
   } else {
     rc = setup_grids<float, float>(d, want);
     if (rc == MCF_OK) rc = setup_tma<float>(d, want);
     if (rc == MCF_OK) rc = setup_resident<float, float>(d, want);
+    if (rc == MCF_OK) rc = setup_flat<float, float>(d, want);
   }
   return rc;
 }
@@ -665,6 +701,7 @@ static int alloc_state(mcf_problem* p, int precision, int device, int shape, cud
   d->device = device;
   d->precision = precision;
   d->renumbered = !p->topo.node_of.empty();
+  d->general_pow = p->kind == MCF_POW && (!p->gamma_mat.empty() || p->gamma_scalar != 0.5);
   d->n = p->n;
   d->m = p->m;
   d->ld = (int)ld_of(p->n);
@@ -815,7 +852,7 @@ static int node_blocks(const DeviceState* d) { return d->tma >= 0 ? d->grid_node
 
 template <typename P, typename S>
 static cudaError_t launch_iteration(DeviceState* d, IterArgs<P, S> a, int parity, bool check,
-                                    cudaStream_t st) {
+                                    cudaStream_t st, int64_t k = -1) {
   const KernelTable<P, S>& T = get_table<P, S>();
   a.parity = parity;
   a.check = check ? 1 : 0;
@@ -830,7 +867,7 @@ static cudaError_t launch_iteration(DeviceState* d, IterArgs<P, S> a, int parity
     if (e != cudaSuccess) return e;
   }
   ScalarArgs sa{d->sc, d->part_edge, edge_blocks(d), d->part_node, node_blocks(d),
-                d->part_check, d->grid_check, check ? 1 : 0};
+                d->part_check, d->grid_check, check ? 1 : 0, k};
   scalar_kernel<<<1, 256, 0, st>>>(sa);
   return cudaGetLastError();
 }
@@ -883,7 +920,7 @@ static cudaError_t launch_iteration_timed(DeviceState* d, IterArgs<P, S> a, int 
     cudaEventRecord(pool.next(2), st);
   }
   ScalarArgs sa{d->sc, d->part_edge, edge_blocks(d), d->part_node, node_blocks(d),
-                d->part_check, d->grid_check, check ? 1 : 0};
+                d->part_check, d->grid_check, check ? 1 : 0, -1};
   scalar_kernel<<<1, 256, 0, st>>>(sa);
   cudaEventRecord(pool.next(3), st);
   return cudaGetLastError();
@@ -1028,6 +1065,30 @@ static cudaError_t launch_resident(DeviceState* d, const IterArgs<P, S>& args, i
   return e;
 }
 
+// Queue iterations [k, k + count): where no scalar tail is needed two launches, the register edge
+// phase and the flat node phase (a graph would save nothing at these durations).
+template <typename P, typename S>
+static cudaError_t launch_flat(DeviceState* d, const IterArgs<P, S>& args, int* parity, int64_t k, int64_t count,
+                               int64_t max_iters, int64_t kc, int64_t k_adapt, cudaStream_t st) {
+  k_adapt = std::max<int64_t>(1, k_adapt);
+  const KernelTable<P, S>& T = get_table<P, S>();
+  cudaError_t e = cudaSuccess;
+  for (const int64_t end = k + count; k < end && e == cudaSuccess; ++k, *parity ^= 1) {
+    const bool check = (k + 1) % kc == 0 || k + 1 >= max_iters;
+    if (check || k % k_adapt == 0) {
+      e = launch_iteration<P, S>(d, args, *parity, check, st, k);
+      continue;
+    }
+    IterArgs<P, S> a = args;
+    a.parity = *parity;
+    void* kargs[] = {&a};
+    e = cudaLaunchKernel((const void*)T.edge[d->shape], dim3(d->grid_edge), dim3(d->block), kargs, 0, st);
+    if (e == cudaSuccess)
+      e = cudaLaunchKernel(flat_kernel<P, S>(), dim3(d->grid_flat), dim3(FLAT_BLOCK), kargs, 0, st);
+  }
+  return e;
+}
+
 // Most iterations of one group of resident launches (whole chunks of k_check): the host looks
 // at the result, and other work gets the GPU, at least this often.
 constexpr int64_t kResidentIters = 1000;
@@ -1135,6 +1196,8 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
       if (!log) chunk = std::min<int64_t>((int64_t)kc * std::max<int64_t>(1, kResidentIters / kc), max_iters - k);
       CK((launch_resident<P, S>(d, args, parity, k, chunk, max_iters, kc, o->k_adapt, stop, st)));
       CK(cudaMemcpyAsync(&stop_state, &d->ctl->stop, sizeof(stop_state), cudaMemcpyDeviceToHost, st));
+    } else if (d->grid_flat > 0 && kt == nullptr) {
+      CK((launch_flat<P, S>(d, args, &parity, k, chunk, max_iters, kc, o->k_adapt, st)));
     } else {
       if (use_graphs && chunk == kc && !stall_first) {
         if (!d->graph[parity] && !capture_chunk<P, S>(d, args, parity, kc, st, &d->graph[parity])) {

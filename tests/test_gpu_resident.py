@@ -1,5 +1,5 @@
-"""The resident iteration (many iterations per launch, automatic shapes with short rows) against
-the oracle, at the edges of its variants: rows that fill a warp's chunks exactly and one entry
+"""The resident iteration (many iterations per launch, automatic shapes with short rows) and the
+flat node phase (longer rows) against the oracle, at the edges of their variants: rows that fill a warp's chunks exactly and one entry
 more, a network served by one CTA, nodes with more than 32 incident edges, a scalar tail in
 every iteration, chunks that do not divide the iteration count, exponents of 1/2 among others;
 and its stop test on the device against the driver's."""
@@ -45,6 +45,10 @@ CASES = [   # (network, precision, iterations, k_check, k_adapt)
     (lambda: _powij(70, 5), "fp32", 25, 10, 100),
     (lambda: I.ring_random_instance(511, 3, 6, "u1_10", "log"), "fp64", 6, 3, 100),
     (lambda: I.ring_random_instance(300, 4, 7, "u1_10", "log"), "bf16", 6, 3, 100),
+    (lambda: I.ring_random_instance(513, 3, 8, "lognormal", "pow", gamma=0.4), "fp64", 8, 4, 100),
+    (lambda: I.ring_random_instance(1025, 3, 9, "u1_10", "log"), "fp32", 7, 5, 100),
+    (lambda: I.ring_random_instance(1025, 3, 9, "lognormal", "pow", gamma=0.5), "bf16", 6, 4, 3),
+    (lambda: I.ring_random_instance(2051, 3, 10, "lognormal", "pow", gamma=0.6), "fp32", 5, 5, 100),
 ]
 
 
