@@ -300,8 +300,7 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
     P delta, tr = P(0);
     if (live) {
       const P vv = x.yo[u] + (x.yl[u] - beta * fplus_at);
-      // (with BF16-stored F a last-place difference of Y flips roundings of F, so that path
-      // keeps the search of node_kernel, to the bit)
+      // (BF16-stored F: node_kernel's search, see setup_resident)
       if (a.kind == 0 || sizeof(S) == 2) tr = prox_traffic<P>(a.kind, vv, beta, x.wv[u], x.gv[u]);
       else prox_pow_traffic<P>(vv, beta, x.wv[u], x.wg[u], x.gv[u], tr);
       delta = -beta * (fplus_at + tr);

@@ -130,6 +130,7 @@ struct DeviceState {
   int requested_shape = -1;   // mcf_options.shape the grids were configured for
   // pipelined edge phase (tma >= 0): one CTA per SM over head-aligned edge ranges
   int tma = -1, tma_kind = 0, grid_tma = 0, grid_node_pin = 0;   // kind 1 bulk-copy, 2 in-sum
+  bool power = false;        // power utility
   bool general_pow = false;  // power utility with an exponent other than 1/2
   bool renumbered = false;   // nodes relabelled for locality (Topology::node_of)
   size_t tma_smem = 0;
@@ -202,7 +203,7 @@ std::mutex g_pool_mu;
 PoolSlot g_pools[kPoolDevices];
 }  // namespace
 
-static cudaMemPool_t state_pool(int device) {
+cudaMemPool_t state_pool(int device) {
   if (device < 0 || device >= kPoolDevices) return nullptr;
   std::lock_guard<std::mutex> g(g_pool_mu);
   PoolSlot& s = g_pools[device];
@@ -546,6 +547,10 @@ template <typename P, typename S>
 static int setup_resident(DeviceState* d, int want) {
   d->resident = -1;
   d->grid_resident = 0;
+  // With BF16-stored F a last-place difference in Y flips roundings of F; log utility's prox gives
+  // the bits of node_kernel, the power search does not, and on small networks that moved the dual
+  // bound by 1e-4. There BF16 keeps the per-phase kernels (see setup_flat for long rows).
+  if (sizeof(S) == 2 && d->power) return MCF_OK;
   const int t = want < 0 && d->tma < 0 ? pick_resident<P, S>((int)(d->ld / StoreTraits<S>::VW)) : -1;
   if (t < 0 || d->ld > 1024) return MCF_OK;   // (BF16, n = 2000: 151 us per-phase, 175 us resident)
   int coop = 0, sms = 0, occ = 0;
@@ -585,7 +590,7 @@ static int setup_flat(DeviceState* d, int want) {
   d->grid_flat = 0;
   if (want >= 0 || d->resident >= 0) return MCF_OK;
   const int most = sizeof(P) == 8 ? INT32_MAX : d->general_pow ? 4096 : d->renumbered ? 1536 : 3584;
-  if (d->ld > most) return MCF_OK;
+  if (d->ld > most || (sizeof(S) == 2 && d->power && d->ld < 2048)) return MCF_OK;
   int sms = 0, occ = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d->device));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (flat_kernel<P, S>()), FLAT_BLOCK, 0));
@@ -701,6 +706,7 @@ static int alloc_state(mcf_problem* p, int precision, int device, int shape, cud
   d->device = device;
   d->precision = precision;
   d->renumbered = !p->topo.node_of.empty();
+  d->power = p->kind == MCF_POW;
   d->general_pow = p->kind == MCF_POW && (!p->gamma_mat.empty() || p->gamma_scalar != 0.5);
   d->n = p->n;
   d->m = p->m;
