@@ -1548,71 +1548,4 @@ check_kernel(IterArgs<P, S> a) {
   block_sum_write<BLOCK, CHECK_PARTS>(acc, a.part_check + (size_t)blockIdx.x * CHECK_PARTS);
 }
 
-// ------------------------------------------------------------------ standalone projection
-// Pi of Sec. 2.3 applied to m columns given as rows of Qt (edge-major, ld >= n floats per
-// row): Ft row l = (q_l - mu_l)_+, mu in/out (warm start in, multipliers out), and the
-// per-column FP64 squared distance ||Pi(q_l) - q_l||^2 into col_d2[l]. Entries n..ld-1 of
-// Qt are ignored; those of Ft are written as zero.
-struct ProjArgs {
-  int n, m, ld;
-  const float* Qt;
-  const float* cap;
-  float* Ft;
-  float* mu;
-  double* col_d2;
-};
-
-template <int VPT, int GROUP, int BLOCK, int MINB>
-__global__ void __launch_bounds__(BLOCK, MINB)
-project_kernel(ProjArgs a) {
-  constexpr int VW = 4;
-  constexpr int GPB = BLOCK / GROUP;
-  __shared__ GroupScratch<GROUP> sh_all[GPB];
-  GroupScratch<GROUP>& sh = sh_all[threadIdx.x / GROUP];
-  int phase = 0;
-  const int lane = threadIdx.x % GROUP;
-  const int gid = blockIdx.x * GPB + threadIdx.x / GROUP;
-  const int ngroups = gridDim.x * GPB;
-  const int nchunks = a.ld / VW;
-  for (int e = gid; e < a.m; e += ngroups) {
-    const float* qr = a.Qt + (size_t)e * a.ld;
-    float q[VPT][VW];
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const int ci = v * GROUP + lane;
-      if (ci < nchunks) {
-        ld_stream<float, VW>(qr + ci * VW, q[v]);
-#pragma unroll
-        for (int u = 0; u < VW; ++u)
-          if (ci * VW + u >= a.n) q[v][u] = 0.f;       // pads never enter the active set
-      } else {
-#pragma unroll
-        for (int u = 0; u < VW; ++u) q[v][u] = 0.f;
-      }
-    }
-    const float mu0 = a.mu[e];
-    const float mu = project_mu<GROUP, VPT, VW, float>(q, a.cap[e], mu0 > 0.f ? mu0 : 0.f, 0.f, sh, phase);
-    float dloc = 0.f;
-#pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-      const int ci = v * GROUP + lane;
-      if (ci < nchunks) {
-        float out[VW];
-#pragma unroll
-        for (int u = 0; u < VW; ++u) {
-          out[u] = q[v][u] > mu ? q[v][u] - mu : 0.f;
-          const float d = out[u] - q[v][u];
-          dloc = fmaf(d, d, dloc);
-        }
-        st_stream<float, VW>(a.Ft + (size_t)e * a.ld + ci * VW, out);
-      }
-    }
-    const double d2 = group_sum_double<GROUP>((double)dloc, sh, phase);
-    if (lane == 0) {
-      a.mu[e] = mu;
-      a.col_d2[e] = d2;
-    }
-  }
-}
-
 }  // namespace pdmcf
