@@ -1,9 +1,9 @@
 // pdmcf_batch.cu — BatchEngine: many resident instances advanced together, and the
 // synchronous batched solve mcf_solve_batch.
 //
-// Per iteration: for every non-empty shape class one edge, one node and one check launch
-// over the class's work list, then one scalar launch with a block per instance. Instance
-// scalars live on the device (BatchScalars), so a chunk of iterations is captured once as a
+// Per iteration: an edge launch over the instances of each non-empty group of shapes, one node
+// and (where some instance takes a stop test) one check launch over all instances, then one
+// scalar launch with a block per instance. Instance scalars live on the device (BatchScalars), so a chunk of iterations is captured once as a
 // CUDA graph and replayed whatever the mix; the host reads the scalar mirror once per chunk
 // to retire finished instances and admit new ones between chunks.
 #include <cuda_runtime.h>
@@ -46,12 +46,28 @@ __global__ void __launch_bounds__(256) batch_scalar_kernel(BatchScalarArgs a) {
   BatchScalars* bs = I.sc;
   if (!bs->active) return;
   const bool check = batch_is_check(bs);
+  const bool reduce = batch_reduces(bs);
+  // without a use for the sums of this iteration only the counters move
+  if (!reduce) {
+    if (threadIdx.x != 0) return;
+    DevScalars* s = &bs->s;
+    s->alpha_last = s->alpha;
+    s->beta_last = s->beta;
+    s->k += 1;
+    bs->parity ^= 1;
+    if (s->numeric_error) {
+      bs->done = 2;
+      bs->active = 0;
+    }
+    return;
+  }
+  const int np = I.n * I.per;
   const double dF2 = det_sum(I.pe, I.m, 1, 0, sh);
-  const double dY2 = det_sum(I.pn, I.n, NODE_PARTS, 0, sh);
+  const double dY2 = det_sum(I.pn, np, NODE_PARTS, 0, sh);
   double nodep[NODE_PARTS];
   double chk[CHECK_PARTS];
   if (check) {
-    for (int f = 1; f < NODE_PARTS; ++f) nodep[f] = det_sum(I.pn, I.n, NODE_PARTS, f, sh);
+    for (int f = 1; f < NODE_PARTS; ++f) nodep[f] = det_sum(I.pn, np, NODE_PARTS, f, sh);
     for (int f = 0; f < CHECK_PARTS; ++f) chk[f] = det_sum(I.pc, I.m, CHECK_PARTS, f, sh);
   }
   if (threadIdx.x != 0) return;
@@ -89,8 +105,11 @@ int batch_admit_shape(const mcf_problem* p) {
   return pick_shape(ld / 4);
 }
 
+static int node_pieces_per(int n) { return batch_pieces_per((n + 7) / 8 * 8); }
+
 int64_t BatchEngine::extra_bytes(const mcf_problem* p) {
-  return (int64_t)sizeof(double) * ((int64_t)p->m * (1 + CHECK_PARTS) + (int64_t)p->n * NODE_PARTS);
+  return (int64_t)sizeof(double) * ((int64_t)p->m * (1 + CHECK_PARTS) +
+                                    (int64_t)p->n * node_pieces_per(p->n) * NODE_PARTS);
 }
 
 BatchEngine::BatchEngine(int device, int max_slots)
@@ -134,23 +153,25 @@ int BatchEngine::init() {
   BCK(cudaMallocHost((void**)&h_sc_, S * sizeof(BatchScalars)));
   BCK(cudaMalloc((void**)&d_slot_list_, S * sizeof(int)));
   BCK(cudaMalloc((void**)&d_nslots_, sizeof(int)));
-  BCK(cudaMalloc((void**)&d_cls_count_, NUM_SHAPES * sizeof(int)));
-  BCK(cudaMalloc((void**)&d_cls_inst_, NUM_SHAPES * S * sizeof(int)));
-  BCK(cudaMalloc((void**)&d_cls_eoff_, NUM_SHAPES * (S + 1) * sizeof(long long)));
-  BCK(cudaMalloc((void**)&d_cls_noff_, NUM_SHAPES * (S + 1) * sizeof(long long)));
+  BCK(cudaMalloc((void**)&d_cls_count_, NUM_LISTS * sizeof(int)));
+  BCK(cudaMalloc((void**)&d_cls_inst_, NUM_LISTS * S * sizeof(int)));
+  BCK(cudaMalloc((void**)&d_cls_eoff_, NUM_LISTS * (S + 1) * sizeof(long long)));
+  BCK(cudaMalloc((void**)&d_cls_noff_, NUM_LISTS * (S + 1) * sizeof(long long)));
   std::memset(h_sc_, 0, S * sizeof(BatchScalars));
   BCK(cudaMemsetAsync(d_sc_, 0, S * sizeof(BatchScalars), stream_));
   BCK(cudaMemsetAsync(d_nslots_, 0, sizeof(int), stream_));
-  BCK(cudaMemsetAsync(d_cls_count_, 0, NUM_SHAPES * sizeof(int), stream_));
+  BCK(cudaMemsetAsync(d_cls_count_, 0, NUM_LISTS * sizeof(int), stream_));
   const BatchTable& T = batch_table();
-  for (int c = 0; c < NUM_SHAPES; ++c) {
-    BatchKernel ks[3] = {T.edge[c], T.node[c], T.check[c]};
-    for (int k = 0; k < 3; ++k) {
-      int occ = 0;
-      BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)ks[k], kShapes[c].block, 0));
-      grid_[k][c] = std::max(1, occ) * sms_;
-    }
-  }
+  auto grid = [&](BatchKernel k, int block, int* out) -> cudaError_t {
+    int occ = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k, block, 0);
+    *out = std::max(1, occ) * sms_;
+    return e;
+  };
+  for (int g = 0; g < NUM_GROUPS; ++g) BCK(grid(T.edge[g], T.block[g], &grid_edge_[g]));
+  BCK(grid(T.node, 256, &grid_node_));
+  BCK(grid(T.node_chk, 256, &grid_node_chk_));
+  BCK(grid(T.check, 256, &grid_check_));
   BCK(cudaStreamSynchronize(stream_));
   return MCF_OK;
 }
@@ -191,7 +212,7 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   auto A = [&](double** ptr, size_t count) {
     return cudaMalloc((void**)ptr, std::max<size_t>(count, 1) * sizeof(double)) == cudaSuccess;
   };
-  if (!A(&sl.pe, p->m) || !A(&sl.pn, (size_t)p->n * NODE_PARTS) ||
+  if (!A(&sl.pe, p->m) || !A(&sl.pn, (size_t)p->n * node_pieces_per(p->n) * NODE_PARTS) ||
       !A(&sl.pc, (size_t)p->m * CHECK_PARTS)) {
     cudaGetLastError();
     for (double* b : {sl.pe, sl.pn, sl.pc})
@@ -201,7 +222,7 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
     return MCF_ERR_OOM;
   }
   BCK(cudaMemsetAsync(sl.pc, 0, (size_t)p->m * CHECK_PARTS * sizeof(double), stream_));
-  BCK(cudaMemsetAsync(sl.pn, 0, (size_t)p->n * NODE_PARTS * sizeof(double), stream_));
+  BCK(cudaMemsetAsync(sl.pn, 0, (size_t)p->n * node_pieces_per(p->n) * NODE_PARTS * sizeof(double), stream_));
   sl.used = true;
   sl.p = p;
   sl.opts = o;
@@ -214,6 +235,7 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   bi.rho = (float)o.rho;
   bi.pe = sl.pe;
   bi.pn = sl.pn;
+  bi.per = node_pieces_per(p->n);
   bi.pc = sl.pc;
   bi.sc = d_sc_ + s;
   h_insts_[s] = bi;
@@ -258,26 +280,28 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   return MCF_OK;
 }
 
-// Class work lists (slot order within a class) and the scalar kernel's slot list.
+// Work lists of the edge-phase groups and of all instances (in slot order) and the scalar
+// kernel's slot list.
 int BatchEngine::upload_lists() {
   const size_t S = max_slots_;
-  std::vector<int> count(NUM_SHAPES, 0), inst(NUM_SHAPES * S, 0), slot_list;
-  std::vector<long long> eoff(NUM_SHAPES * (S + 1), 0), noff(NUM_SHAPES * (S + 1), 0);
+  std::vector<int> count(NUM_LISTS, 0), inst(NUM_LISTS * S, 0), slot_list;
+  std::vector<long long> eoff(NUM_LISTS * (S + 1), 0), noff(NUM_LISTS * (S + 1), 0);
   unsigned mask = 0;
   for (int s = 0; s < max_slots_; ++s) {
     const BatchSlot& sl = slots_[s];
     if (!sl.used || sl.finished) continue;
-    const int c = sl.cls;
-    const int k = count[c]++;
-    inst[c * S + k] = s;
-    eoff[c * (S + 1) + k + 1] = eoff[c * (S + 1) + k] + sl.p->m;
-    noff[c * (S + 1) + k + 1] = noff[c * (S + 1) + k] + sl.p->n;
+    for (int c : {batch_group(sl.cls), NUM_GROUPS}) {
+      const int k = count[c]++;
+      inst[c * S + k] = s;
+      eoff[c * (S + 1) + k + 1] = eoff[c * (S + 1) + k] + sl.p->m;
+      noff[c * (S + 1) + k + 1] = noff[c * (S + 1) + k] + (long long)sl.p->n * h_insts_[s].per;
+    }
     slot_list.push_back(s);
-    mask |= 1u << c;
+    mask |= 1u << batch_group(sl.cls);
   }
   const int ns = (int)slot_list.size();
   if (slot_list.empty()) slot_list.push_back(0);
-  BCK(cudaMemcpyAsync(d_cls_count_, count.data(), NUM_SHAPES * sizeof(int), cudaMemcpyHostToDevice, stream_));
+  BCK(cudaMemcpyAsync(d_cls_count_, count.data(), NUM_LISTS * sizeof(int), cudaMemcpyHostToDevice, stream_));
   BCK(cudaMemcpyAsync(d_cls_inst_, inst.data(), inst.size() * sizeof(int), cudaMemcpyHostToDevice, stream_));
   BCK(cudaMemcpyAsync(d_cls_eoff_, eoff.data(), eoff.size() * sizeof(long long), cudaMemcpyHostToDevice, stream_));
   BCK(cudaMemcpyAsync(d_cls_noff_, noff.data(), noff.size() * sizeof(long long), cudaMemcpyHostToDevice, stream_));
@@ -292,18 +316,17 @@ int BatchEngine::upload_lists() {
 int BatchEngine::launch_iteration(cudaStream_t st, bool with_check) {
   const BatchTable& T = batch_table();
   const size_t S = max_slots_;
-  for (int c = 0; c < NUM_SHAPES; ++c) {
-    if (!(class_mask_ & (1u << c))) continue;
-    BatchClassDev cls{d_cls_count_ + c, d_cls_inst_ + c * S, d_cls_eoff_ + c * (S + 1),
-                      d_cls_noff_ + c * (S + 1)};
-    const BatchInst* insts = d_insts_;
+  const BatchInst* insts = d_insts_;
+  auto launch = [&](BatchKernel k, int list, int grid, int block) -> cudaError_t {
+    BatchClassDev cls{d_cls_count_ + list, d_cls_inst_ + list * S, d_cls_eoff_ + list * (S + 1),
+                      d_cls_noff_ + list * (S + 1)};
     void* kargs[] = {(void*)&insts, &cls};
-    const int block = kShapes[c].block;
-    BCK(cudaLaunchKernel((const void*)T.edge[c], dim3(grid_[0][c]), dim3(block), kargs, 0, st));
-    BCK(cudaLaunchKernel((const void*)T.node[c], dim3(grid_[1][c]), dim3(block), kargs, 0, st));
-    if (with_check)
-      BCK(cudaLaunchKernel((const void*)T.check[c], dim3(grid_[2][c]), dim3(block), kargs, 0, st));
-  }
+    return cudaLaunchKernel((const void*)k, dim3(grid), dim3(block), kargs, 0, st);
+  };
+  for (int g = 0; g < NUM_GROUPS; ++g)
+    if (class_mask_ & (1u << g)) BCK(launch(T.edge[g], g, grid_edge_[g], T.block[g]));
+  BCK(launch(with_check ? T.node_chk : T.node, NUM_GROUPS, with_check ? grid_node_chk_ : grid_node_, 256));
+  if (with_check) BCK(launch(T.check, NUM_GROUPS, grid_check_, 256));
   BatchScalarArgs sa{d_insts_, d_slot_list_, d_nslots_};
   batch_scalar_kernel<<<max_slots_, 256, 0, st>>>(sa);
   BCK(cudaGetLastError());
@@ -483,6 +506,8 @@ int tune_class(int device, int c0) {
   std::vector<int> cands;
   for (int s = 0; s < NUM_SHAPES; ++s) {
     const int cap = kShapes[s].group * kShapes[s].vpt;
+    // (shapes of one group are one kernel)
+    if (s != c0 && batch_group(s) == batch_group(c0)) continue;
     if (cap >= cap0 && cap <= 4 * cap0) cands.push_back(s);
   }
   constexpr int kCount = 16;

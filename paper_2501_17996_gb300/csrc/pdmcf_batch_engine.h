@@ -15,10 +15,15 @@
 namespace pdmcf {
 
 using BatchKernel = void (*)(const BatchInst*, BatchClassDev);
+// Edge-phase launches: shapes with a warp per edge share one for rows of up to 512 entries and
+// one for up to 1024, each longer shape has its own. Node phase and check serve all instances.
+constexpr int NUM_GROUPS = 2 + NUM_SHAPES - 4;
+constexpr int batch_group(int shape) { return shape < 3 ? 0 : shape == 3 ? 1 : shape - 2; }
+static_assert(kShapes[3].group == 32 && kShapes[4].group > 32, "the first four shapes are warp shapes");
 struct BatchTable {
-  BatchKernel edge[NUM_SHAPES];
-  BatchKernel node[NUM_SHAPES];
-  BatchKernel check[NUM_SHAPES];
+  BatchKernel edge[NUM_GROUPS];
+  int block[NUM_GROUPS];
+  BatchKernel node, node_chk, check;   // 256 threads
 };
 const BatchTable& batch_table();
 
@@ -76,11 +81,14 @@ class BatchEngine {
   BatchScalars* h_sc_ = nullptr;       // pinned mirror
   int* d_slot_list_ = nullptr;
   int* d_nslots_ = nullptr;
-  int* d_cls_count_ = nullptr;          // [NUM_SHAPES]
-  int* d_cls_inst_ = nullptr;           // [NUM_SHAPES * max_slots]
-  long long* d_cls_eoff_ = nullptr;     // [NUM_SHAPES * (max_slots + 1)]
+  // work lists of the edge-phase launches and, at NUM_GROUPS, of all instances
+  int* d_cls_count_ = nullptr;          // [NUM_LISTS]
+  int* d_cls_inst_ = nullptr;           // [NUM_LISTS * max_slots]
+  long long* d_cls_eoff_ = nullptr;     // [NUM_LISTS * (max_slots + 1)]
   long long* d_cls_noff_ = nullptr;
-  int grid_[3][NUM_SHAPES] = {};
+  static constexpr int NUM_LISTS = NUM_GROUPS + 1;
+  int grid_edge_[NUM_GROUPS] = {};
+  int grid_node_ = 0, grid_node_chk_ = 0, grid_check_ = 0;
   std::vector<BatchSlot> slots_;
   std::vector<BatchInst> h_insts_;
   bool lists_dirty_ = true;

@@ -237,7 +237,9 @@ __device__ __forceinline__ void node_state(const IterArgs<P, S>& a, int par, con
 // R of the node's rows, k.. of the 32 whose edges the lanes hold, added to s with their signs.
 // The loads are unconditional (rows past the last repeat it with weight 0), so that all R are in
 // flight at once.
-template <typename P, typename S, int N, int R>
+// PAIRS: rounded as node_kernel rounds it, consecutive rows added as pairs; else one row after the
+// other (the batched engine's order).
+template <typename P, typename S, int N, int R, bool PAIRS>
 __device__ __forceinline__ void node_rows(const S* __restrict__ f0, size_t ld, int edge, int k, int nin, int deg,
                                           P (&s)[N]) {
   S f[R][N];
@@ -245,16 +247,20 @@ __device__ __forceinline__ void node_rows(const S* __restrict__ f0, size_t ld, i
   for (int r = 0; r < R; ++r)
     ld_words<S, N>(f0 + (size_t)__shfl_sync(0xffffffffu, edge, k + r) * ld, f[r]);
 #pragma unroll
-  for (int r = 0; r < R; r += 2) {   // consecutive pairs, as node_kernel adds them
+  for (int r = 0; r < R; r += 2) {
     const P s0 = k + r < nin ? P(1) : k + r < deg ? P(-1) : P(0);
     const P s1 = k + r + 1 < nin ? P(1) : k + r + 1 < deg ? P(-1) : P(0);
 #pragma unroll
-    for (int u = 0; u < N; ++u) s[u] += fma(s0, to_p<P>(f[r][u]), s1 * to_p<P>(f[r + 1][u]));
+    for (int u = 0; u < N; ++u) {
+      const P x0 = to_p<P>(f[r][u]), x1 = to_p<P>(f[r + 1][u]);
+      if constexpr (PAIRS) s[u] += fma(s0, x0, s1 * x1);
+      else s[u] = fma(s1, x1, fma(s0, x0, s[u]));
+    }
   }
 }
 
 // s = sum_{in(j)} f - sum_{out(j)} f over the lane's N entries.
-template <typename P, typename S, int N>
+template <typename P, typename S, int N, bool PAIRS = true>
 __device__ __forceinline__ void node_gather(const IterArgs<P, S>& a, const S* __restrict__ Fn,
                                             const NodePiece& q, P (&s)[N]) {
   const S* f0 = Fn + (q.c * N < a.ld ? (size_t)q.c * N : 0);
@@ -267,18 +273,18 @@ __device__ __forceinline__ void node_gather(const IterArgs<P, S>& a, const S* __
     const int nin = q.nin - b, deg = q.deg - b, cnt = min(32, deg);
     int k = 0;
     if (N == 1 && cnt > 16) {
-      node_rows<P, S, N, 24>(f0, a.ld, edge, 0, nin, deg, s);
+      node_rows<P, S, N, 24, PAIRS>(f0, a.ld, edge, 0, nin, deg, s);
       k = 24;
     } else if (N <= 2 && cnt > 12) {
-      node_rows<P, S, N, 16>(f0, a.ld, edge, 0, nin, deg, s);
+      node_rows<P, S, N, 16, PAIRS>(f0, a.ld, edge, 0, nin, deg, s);
       k = 16;
     }
     if constexpr (N > 2) {
 #pragma unroll 1
-      for (; k + 6 < cnt; k += 8) node_rows<P, S, N, 8>(f0, a.ld, edge, k, nin, deg, s);
+      for (; k + 6 < cnt; k += 8) node_rows<P, S, N, 8, PAIRS>(f0, a.ld, edge, k, nin, deg, s);
     }
 #pragma unroll 1
-    for (; k < cnt; k += 4) node_rows<P, S, N, 4>(f0, a.ld, edge, k, nin, deg, s);
+    for (; k < cnt; k += 4) node_rows<P, S, N, 4, PAIRS>(f0, a.ld, edge, k, nin, deg, s);
   }
 }
 
