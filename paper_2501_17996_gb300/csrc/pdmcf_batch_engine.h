@@ -34,9 +34,7 @@ struct BatchSlot {
   mcf_options opts{};
   void* tag = nullptr;
   int cls = -1;
-  double* pe = nullptr;
-  double* pn = nullptr;
-  double* pc = nullptr;
+  double* parts = nullptr;   // pe, pn and pc of its BatchInst
   int64_t bytes = 0;
   bool finished = false;
   int status = MCF_PENDING;
@@ -60,12 +58,14 @@ class BatchEngine {
   int step(int iters);
   // Finished slots since the last call.
   std::vector<int> take_finished();
-  // Copy the slot's final state back into its problem and free the slot.
-  void release(int slot);
+  // Copy the slot's final state back into its problem and free the slot. The state may be used
+  // on other streams once the engine's has been waited for: by this call or a later one with wait.
+  void release(int slot, bool wait = true);
   const BatchSlot& slot(int s) const { return slots_[s]; }
   static int64_t extra_bytes(const mcf_problem* p);   // engine buffers per instance
 
  private:
+  double* alloc_parts(size_t bytes);
   int step_impl(int iters);
   int upload_lists();
   int launch_iteration(cudaStream_t st, bool with_check);
@@ -75,6 +75,7 @@ class BatchEngine {
   int device_;
   int max_slots_;
   cudaStream_t stream_ = nullptr;
+  cudaMemPool_t pool_ = nullptr;        // of the problems' states; nullptr: plain allocations
   int sms_ = 0;
   BatchInst* d_insts_ = nullptr;
   BatchScalars* d_sc_ = nullptr;

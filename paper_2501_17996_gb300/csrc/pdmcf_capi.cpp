@@ -332,7 +332,7 @@ int mcf_update_weights(mcf_problem* p, const double* w) {
   if (rc != MCF_OK) return rc;
   std::lock_guard<std::mutex> g(p->lock);
   p->w.swap(wcopy);
-  p->data_dirty = true;
+  p->data_dirty = p->weights_dirty = true;
   return MCF_OK;
 }
 

@@ -103,6 +103,7 @@ struct mcf_problem {
   double eta = 0.0;
   double omega = 1.0;                  // resident primal weight (warm start)
   bool data_dirty = true;              // cap / w changed since the last upload
+  bool weights_dirty = true;           // among them w (or a new state without w and gamma)
   pdmcf::DeviceState* ds = nullptr;
   std::mutex lock;                     // one call at a time per problem
   std::atomic<int> busy{0};            // >0 while a ticket uses the problem

@@ -401,7 +401,9 @@ static int chunk_rows(int n, int cols) {
   return (int)std::max<size_t>(32, std::min<size_t>((size_t)n, ((size_t)64 << 20) / per));
 }
 
-// Upload c and w (placed as Wt[node(j)][node(i)] = w_ij) and per-pair gamma in precision P.
+// Upload c and, unless only c has changed since the last upload, w (placed as
+// Wt[node(j)][node(i)] = w_ij) and per-pair gamma in precision P. After a change of the capacities
+// alone w is n^2 doubles that the device has already: n = 10^4, 800 MB, 35 ms of a re-solve.
 template <typename P>
 static int upload_data(mcf_problem* p, DeviceState* d, cudaStream_t st) {
   const int n = p->n, m = p->m;
@@ -409,6 +411,11 @@ static int upload_data(mcf_problem* p, DeviceState* d, cudaStream_t st) {
   std::vector<P> cap(m);
   for (int e = 0; e < m; ++e) cap[e] = (P)p->cap[p->topo.perm[e]];
   CK(cudaMemcpyAsync(d->cap, cap.data(), m * sizeof(P), cudaMemcpyHostToDevice, st));
+  if (!p->weights_dirty) {
+    CK(cudaStreamSynchronize(st));   // the host vector
+    p->data_dirty = false;
+    return MCF_OK;
+  }
   int rc = ensure_node_map(p, d, st);
   if (rc != MCF_OK) return rc;
   const int rows = chunk_rows(n, n);
@@ -436,7 +443,7 @@ static int upload_data(mcf_problem* p, DeviceState* d, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the stage and the host vectors
   sfree(d, stage, st);
   CK(e);
-  p->data_dirty = false;
+  p->data_dirty = p->weights_dirty = false;
   return MCF_OK;
 }
 
@@ -783,7 +790,7 @@ static int alloc_state(mcf_problem* p, int precision, int device, int shape, cud
   CK(cudaStreamSynchronize(st));
   rc = upload_cta_ranges(p, d, st);
   if (rc != MCF_OK) { free_state(d); return rc; }
-  p->data_dirty = true;
+  p->data_dirty = p->weights_dirty = true;
   *out = d;
   return MCF_OK;
 }
@@ -1400,13 +1407,13 @@ static int transfer_to_fp32(mcf_problem* p, const mcf_options* o, cudaStream_t s
   dst->lo_live = src->lo_live;
   free_state(src);
   p->ds = dst;
-  p->data_dirty = true;
+  p->data_dirty = p->weights_dirty = true;
   return MCF_OK;
 }
 
 // ------------------------------------------------------------------ batched-engine hooks
 
-// FP32 state on o->device for a batched run: cold start (F = 0, Y = I - 11^T, P = 0,
+// FP32 state on o->device for a batched run, prepared in st's order: cold start (F = 0, Y = I - 11^T, P = 0,
 // mu = 0, omega = omega0) unless a warm start is asked for and an iterate is resident.
 int batch_prepare_state(mcf_problem* p, const mcf_options* o, cudaStream_t st, bool* warm) {
   if (p->ds && (p->ds->precision != MCF_FP32 || p->ds->device != o->device)) device_free(p);
@@ -1437,7 +1444,6 @@ int batch_prepare_state(mcf_problem* p, const mcf_options* o, cudaStream_t st, b
     CK(cudaGetLastError());
     p->omega = o->omega0 > 0 ? o->omega0 : 1.0;
   }
-  CK(cudaStreamSynchronize(st));
   d->valid = false;   // the iterate is in flux until the engine hands it back
   return MCF_OK;
 }
@@ -1472,14 +1478,14 @@ void batch_state_pointers(mcf_problem* p, BatchInst* bi, int* parity) {
   bi->Yhat = (float*)d->Yhat;
 }
 
-// The engine's final scalars become the problem's resident state (warm starts, outputs).
+// The engine's final scalars become the problem's resident state (warm starts, outputs) once st
+// has been synchronised.
 void batch_finish_state(mcf_problem* p, int parity, const DevScalars& s, cudaStream_t st) {
   DeviceState* d = p->ds;
   d->cur = parity;
   d->valid = true;
   p->omega = s.omega;
   cudaMemcpyAsync(d->sc, &s, sizeof(DevScalars), cudaMemcpyHostToDevice, st);
-  cudaStreamSynchronize(st);
 }
 
 // ------------------------------------------------------------------ warm-state checkpoint
