@@ -80,7 +80,9 @@ typedef struct mcf_options {
   int     precision;         /* MCF_FP32 | MCF_FP64 | MCF_BF16_F (default MCF_FP32)         */
   int     warm_start;        /* 1: start from the problem's resident (F, Y, omega)          */
   int     polish_iters;      /* MCF_BF16_F: extra FP32 iterations after convergence         */
-  int     use_graphs;        /* capture each k_check-iteration chunk in a CUDA graph (1)    */
+  int     use_graphs;        /* capture each k_check-iteration chunk in a CUDA graph (1); a
+                                solve whose rows are short enough for the resident
+                                iteration (many iterations per launch) needs none          */
   int     device;            /* CUDA device ordinal (default 0)                             */
   void*   cuda_stream;       /* cudaStream_t to run on; NULL = the library's own stream     */
   double  omega0;            /* initial primal weight for cold starts (default 1.0)         */
@@ -97,7 +99,9 @@ typedef struct mcf_options {
                                 instances of that size (default 1)                         */
   int     shape;             /* kernel launch shape index (-1 = automatic); see
                                 mcf_shape_info. Lets tests and the tuner pick any shape
-                                whose capacity covers the problem                          */
+                                whose capacity covers the problem. A shape named here runs
+                                one launch per phase; -1 may run the resident iteration
+                                (rows of up to 1024 entries) or the flat node phase        */
   double  adapt_guard;       /* g: stop adapting omega (keep it constant, Sec. 2.4) from
                                 the iteration after a stop test where omega is more than a
                                 factor g^2 away from its value at the first stop test with
@@ -209,10 +213,11 @@ void mcf_options_default(mcf_options* o);
  * MCF_ERR_NUMERIC, MCF_ERR_OOM, MCF_ERR_CUDA or MCF_ERR_INVALID. */
 int mcf_solve(mcf_problem* p, const mcf_options* opts, mcf_result* res);
 
-/* Solve `count` independent problems together on one GPU (FP32 iterates only): each PDHG
- * phase is one launch per launch-shape class for all resident problems, every problem keeps
+/* Solve `count` independent problems together on one GPU (FP32 iterates only): the edge phase
+ * is one launch per group of launch shapes and the other phases one launch each for all
+ * resident problems, every problem keeps
  * its own step sizes, iteration count and stop test on the device, and its reductions are
- * summed per edge and per node in a fixed order, so a problem's iterates are identical
+ * summed per edge and per piece of a node's column in a fixed order, so a problem's iterates are identical
  * whether it is solved alone or in any batch. opts applies to every problem (warm_start = 1
  * continues each problem's resident iterate). results[i] is filled as by mcf_solve for
  * problems[i], including any output buffers it points to. The problems must be distinct
@@ -274,8 +279,9 @@ typedef struct mcf_kernel_times {
   int     shape;         /* launch shape the solve used (an mcf_shape_info index)     */
 } mcf_kernel_times;
 
-/* As mcf_solve, but launches every kernel individually (no CUDA graphs) with a CUDA event
- * before and after it on the solve stream, and fills *kt. For measurement. */
+/* As mcf_solve, but launches every kernel of every phase individually (no CUDA graphs, no
+ * resident iteration, the register node phase) with a CUDA event before and after it on the
+ * solve stream, and fills *kt. For measurement. */
 int mcf_solve_timed(mcf_problem* p, const mcf_options* opts, mcf_result* res,
                     mcf_kernel_times* kt);
 
@@ -297,8 +303,8 @@ int mcf_solve_timed(mcf_problem* p, const mcf_options* opts, mcf_result* res,
  *   dist2  host, may be NULL: receives sum_l ||Ft_l - q_l||^2, an FP64 reduction in a fixed
  *          order (independent of the launch grid)
  *   stream cudaStream_t (NULL = legacy default stream), on the calling thread's current device
- * Allocates m+1 doubles of device scratch for the call and synchronizes the stream before
- * returning. Errors: MCF_ERR_INVALID (sizes, NULL or misaligned pointers), MCF_ERR_OOM,
+ * With dist2, m+1 doubles of device scratch come from the pool that also holds the problems'
+ * states, in stream order. Synchronizes the stream before returning. Errors: MCF_ERR_INVALID (sizes, NULL or misaligned pointers), MCF_ERR_OOM,
  * MCF_ERR_CUDA. */
 int mcf_project_capped_simplex(int32_t n, int32_t m, int32_t ld, const float* Qt,
                                const float* cap, float* Ft, float* mu, double* dist2,
