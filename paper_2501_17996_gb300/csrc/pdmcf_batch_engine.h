@@ -49,6 +49,7 @@ class BatchEngine {
   ~BatchEngine();
   int init();                         // allocate the tables; MCF_OK or an error
   int device() const { return device_; }
+  cudaStream_t stream() const { return stream_; }
   int free_slots() const;
   int active_count() const;
   // Admit an FP32 request: allocates/initialises the instance state (cold or warm).
@@ -62,7 +63,7 @@ class BatchEngine {
   // on other streams once the engine's has been waited for: by this call or a later one with wait.
   void release(int slot, bool wait = true);
   const BatchSlot& slot(int s) const { return slots_[s]; }
-  static int64_t extra_bytes(const mcf_problem* p);   // engine buffers per instance
+  static int64_t extra_bytes(const mcf_problem* p);   // engine buffers per instance, as admission counts them
 
  private:
   double* alloc_parts(size_t bytes);

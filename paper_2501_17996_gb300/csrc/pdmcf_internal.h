@@ -114,7 +114,8 @@ int validate_options(const mcf_options* o);   // pdmcf_capi.cpp
 // Implemented in pdmcf_solver.cu.
 int device_solve(mcf_problem* p, const mcf_options* o, mcf_result* res,
                  mcf_kernel_times* kt = nullptr);
-int device_copy_outputs(mcf_problem* p, mcf_result* res);
+// cuda_stream: the state was last written on it (NULL: the problem's own stream, after a wait).
+int device_copy_outputs(mcf_problem* p, mcf_result* res, void* cuda_stream = nullptr);
 int device_save_state(mcf_problem* p, const char* path);
 int device_load_state(mcf_problem* p, const char* path, int device);
 void device_free(mcf_problem* p);

@@ -1360,14 +1360,14 @@ extern "C" int mcf_shape_info(int* group, int* vpt, int* block, int* kind) {
 
 namespace pdmcf {
 
-int device_copy_outputs(mcf_problem* p, mcf_result* res) {
+int device_copy_outputs(mcf_problem* p, mcf_result* res, void* cuda_stream) {
   DeviceState* d = p->ds;
   if (!d || !d->valid) {
     set_error("no solution resident on the device");
     return MCF_ERR_INVALID;
   }
   CK(cudaSetDevice(d->device));
-  cudaStream_t st = d->own_stream;
+  cudaStream_t st = cuda_stream ? (cudaStream_t)cuda_stream : d->own_stream;
   if (d->precision == MCF_FP64) return copy_outputs_t<double, double>(p, d, res, st);
   if (d->precision == MCF_BF16_F) return copy_outputs_t<float, __nv_bfloat16>(p, d, res, st);
   return copy_outputs_t<float, float>(p, d, res, st);
