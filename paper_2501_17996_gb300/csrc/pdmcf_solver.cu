@@ -555,8 +555,8 @@ static int setup_resident(DeviceState* d, int want) {
   d->resident = -1;
   d->grid_resident = 0;
   // With BF16-stored F a last-place difference in Y flips roundings of F; log utility's prox gives
-  // the bits of node_kernel, the power search does not, and on small networks that moved the dual
-  // bound by 1e-4. There BF16 keeps the per-phase kernels (see setup_flat for long rows).
+  // the bits of node_kernel, the power search does not. With power utility BF16 keeps the
+  // per-phase kernels at every length (see setup_flat).
   if (sizeof(S) == 2 && d->power) return MCF_OK;
   const int t = want < 0 && d->tma < 0 ? pick_resident<P, S>((int)(d->ld / StoreTraits<S>::VW)) : -1;
   if (t < 0 || d->ld > 1024) return MCF_OK;   // (BF16, n = 2000: 151 us per-phase, 175 us resident)
@@ -587,17 +587,22 @@ template <> const void* flat_kernel<double, double>() { return (const void*)flat
 // Iterations without a scalar tail on automatic shapes that are not resident: the register edge
 // phase and the flat node phase, against the kernels of setup_grids / setup_tma (us per iteration,
 // GB300, out-degree 8 log or 10 power). FP64: n = 700 393 -> 364, with an exponent per pair
-// 1314 -> 638. Networks without node locality: n = 1500 87 -> 83, n = 2500 299 -> 221 (FP32) and
-// 276 -> 188 (BF16), n = 3500 459 -> 427, n = 4000 power 661 -> 689 (the in-sum kind stays).
+// 1314 -> 638. Networks without node locality: n = 1500 87 -> 83, n = 2500 299 -> 221,
+// n = 3500 459 -> 427, n = 4000 power 661 -> 689 (the in-sum kind stays).
 // Renumbered networks, where the node phase's rows are close in memory anyway: n = 1500 113 -> 111,
 // n = 2000 178 -> 184. With exponents other than 1/2 the flat phase's root search decides:
 // n = 3000 559 -> 426.
+// BF16-stored F takes this path only where it gives the bits of the kernels it stands for: the
+// register shapes (the in-sum kind adds a node's in-edges in another order) with log utility (the
+// power search rounds differently). One last-place difference in Y or in a multiplier flips
+// roundings of F to BF16, each 2^-8 of an entry, and the flips spread: n = 3001, power, 100
+// iterations, T was 2.7e-3 (norm) from the per-phase kernels' with it.
 template <typename P, typename S>
 static int setup_flat(DeviceState* d, int want) {
   d->grid_flat = 0;
   if (want >= 0 || d->resident >= 0) return MCF_OK;
   const int most = sizeof(P) == 8 ? INT32_MAX : d->general_pow ? 4096 : d->renumbered ? 1536 : 3584;
-  if (d->ld > most || (sizeof(S) == 2 && d->power && d->ld < 2048)) return MCF_OK;
+  if (d->ld > most || (sizeof(S) == 2 && (d->power || d->tma >= 0))) return MCF_OK;
   int sms = 0, occ = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d->device));
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (flat_kernel<P, S>()), FLAT_BLOCK, 0));
