@@ -45,9 +45,9 @@ __global__ void __launch_bounds__(256) batch_scalar_kernel(BatchScalarArgs a) {
   if ((int)blockIdx.x >= *a.nslots) return;
   const BatchInst& I = a.insts[a.slots[blockIdx.x]];
   BatchScalars* bs = I.sc;
-  if (!bs->active) return;
-  const bool check = batch_is_check(bs);
-  const bool reduce = batch_reduces(bs);
+  const bool active = bs->active != 0, check = batch_is_check(bs), reduce = batch_reduces(bs);
+  __syncthreads();   // all threads have read the scalars: from here on thread 0 moves them
+  if (!active) return;
   // without a use for the sums of this iteration only the counters move
   if (!reduce) {
     if (threadIdx.x != 0) return;
