@@ -380,6 +380,15 @@ int mcf_load_state(mcf_problem* p, const char* path, int device);
  * invalid, so the next solve starts cold. The paper has no counterpart. Returns MCF_OK. */
 int mcf_test_withhold_next_copy(void);
 
+/* Exercise the bounded waits of the resident iteration's grid barrier: the next solve on the
+ * calling process that runs the resident iteration (automatic shape, rows of up to 1024
+ * entries) waits at its first barrier for one arrival more than there are CTAs. Every CTA gives
+ * up after 2^21 polls (a second or two) and leaves, the launches queued behind return at once,
+ * and the solve ends with MCF_ERR_CUDA ("a bounded device-side wait timed out"). The problem's
+ * iterate is then invalid, so the next solve starts cold. The paper has no counterpart. Returns
+ * MCF_OK. */
+int mcf_test_withhold_next_arrival(void);
+
 /* Message for the last error of the calling thread ("" if none). */
 const char* mcf_last_error(void);
 

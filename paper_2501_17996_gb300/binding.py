@@ -74,6 +74,7 @@ SYMBOLS = [
     "mcf_submit", "mcf_poll", "mcf_wait",
     "mcf_cancel", "mcf_serving_config", "mcf_serving_shutdown", "mcf_project_capped_simplex",
     "mcf_project_capped_simplex_noalloc", "mcf_shape_info", "mcf_test_withhold_next_copy",
+    "mcf_test_withhold_next_arrival",
     "mcf_save_state", "mcf_load_state",
     "mcf_last_error", "mcf_version",
 ]
@@ -113,6 +114,7 @@ def _load() -> C.CDLL:
         "mcf_serving_config": (C.c_int, [C.c_int64, C.c_int]),
         "mcf_serving_shutdown": (C.c_int, []),
         "mcf_test_withhold_next_copy": (C.c_int, []),
+        "mcf_test_withhold_next_arrival": (C.c_int, []),
         "mcf_save_state": (C.c_int, [P, C.c_char_p]),
         "mcf_load_state": (C.c_int, [P, C.c_char_p, C.c_int]),
         "mcf_project_capped_simplex": (C.c_int, [C.c_int32, C.c_int32, C.c_int32, P, P, P, P,
@@ -379,6 +381,14 @@ def mcf_test_withhold_next_copy() -> None:
     rc = LIB.mcf_test_withhold_next_copy()
     if rc != MCF_OK:
         raise MCFError(rc, "mcf_test_withhold_next_copy")
+
+
+def mcf_test_withhold_next_arrival() -> None:
+    """Testing aid: the next resident solve waits for an arrival that never comes, so its first
+    grid barrier runs out of polls."""
+    rc = LIB.mcf_test_withhold_next_arrival()
+    if rc != MCF_OK:
+        raise MCFError(rc, "mcf_test_withhold_next_arrival")
 
 
 def mcf_serving_shutdown() -> None:

@@ -71,8 +71,9 @@ __device__ __forceinline__ void st_tail(__nv_bfloat16* p, const float (&v)[N]) {
 
 // ------------------------------------------------------------------ grid barrier
 // Counter barrier over the CTAs of a cooperative launch, split in arrive and wait. The waits
-// are bounded (2^23 polls, several seconds): a CTA that gives up records wait_timeout and
-// leaves, the others run out of polls the same way, and the driver reports MCF_ERR_CUDA.
+// are bounded (2^21 polls, a second or two): a CTA that gives up records wait_timeout and
+// leaves, the others run out of polls the same way, the launches queued behind this one return
+// at once (resident_start), and the driver reports MCF_ERR_CUDA.
 struct GridBarrier {
   unsigned* arrived;
   DevScalars* sc;
@@ -88,7 +89,7 @@ struct GridBarrier {
     if (threadIdx.x == 0) {
       unsigned v = 0;
       bool ok = false;
-      for (int it = 0; it < (1 << 23) && !ok; ++it) {
+      for (int it = 0; it < (1 << 21) && !ok; ++it) {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
         ok = (int)(v - target) >= 0;
       }
@@ -700,6 +701,14 @@ __device__ __forceinline__ ResidentPlace resident_place(int n, int m, int ld, in
   return w;
 }
 
+// Start of a launch, in thread 0 and before a barrier of the CTA: whether a wait of an earlier launch
+// of the group has run out. That launch left the count of arrivals short, so every barrier behind
+// it would run out of polls as well.
+template <typename P, typename S>
+__device__ __forceinline__ void resident_start(const IterArgs<P, S>& a, int& failed) {
+  if (threadIdx.x == 0) failed = __ldcg(&a.sc->wait_timeout);
+}
+
 // Iterations without a scalar tail. No function call and no spilled register is in the loop: a
 // spilled register would be read back through L2, since every barrier drops the L1.
 template <typename P, typename S, int VPT, int N, int BLOCK>
@@ -718,8 +727,9 @@ resident_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant_
     piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
     node_data<P, S, N>(a, piece, x);
   }
-  if (threadIdx.x == 0) failed = 0;
+  resident_start(a, failed);
   __syncthreads();
+  if (failed) return;
   GridBarrier bar{&ra.ctl->arrived, a.sc, &failed, ra.arrived};
   int par = a.parity;
 #pragma unroll 1
@@ -753,8 +763,9 @@ resident_special_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_c
   __shared__ int failed;
   if (__ldcg(&ra.ctl->stop.verdict) != STOP_NO) return;
   const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N);
-  if (threadIdx.x == 0) failed = 0;
+  resident_start(a, failed);
   __syncthreads();
+  if (failed) return;
   GridBarrier bar{&ra.ctl->arrived, a.sc, &failed, ra.arrived};
   int par = a.parity;
 #pragma unroll 1

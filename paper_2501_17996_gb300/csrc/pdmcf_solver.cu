@@ -1047,25 +1047,33 @@ static void write_check_line(FILE* f, const DevScalars& h, int n, int m, int pre
 static std::atomic<int> g_withhold_request{0};
 static bool take_withhold_request() { return g_withhold_request.exchange(0) != 0; }
 
+// mcf_test_withhold_next_arrival: one pending request, taken by the next resident solve.
+static std::atomic<int> g_withhold_arrival{0};
+
+// Most iterations of one resident launch, and of one group of launches between two looks of the host
+// at the result (there rounded to whole chunks of k_check, at least one).
+constexpr int64_t kResidentIters = 1000;
+
 // Queue iterations [k, k + count) of the resident path: launches of plain iterations between
 // those with a scalar tail (k a multiple of k_adapt, or a stop test). Once a stop test holds on
-// the device the launches behind it return at once.
+// the device, or a barrier has run out of polls, the launches behind it return at once.
+// `withhold`: testing aid, the barriers wait for one arrival that never comes.
 template <typename P, typename S>
 static cudaError_t launch_resident(DeviceState* d, const IterArgs<P, S>& args, int parity, int64_t k, int64_t count,
                                    int64_t max_iters, int64_t kc, int64_t k_adapt, const StopRule& rule,
-                                   cudaStream_t st) {
+                                   bool withhold, cudaStream_t st) {
   const ResidentTable<P, S>& T = get_resident<P, S>();
   k_adapt = std::max<int64_t>(1, k_adapt);
   auto check = [&](int64_t i) { return (i + 1) % kc == 0 || i + 1 >= max_iters; };
   auto special = [&](int64_t i) { return check(i) || i % k_adapt == 0; };
   cudaError_t e = cudaMemsetAsync(&d->ctl->arrived, 0, sizeof(unsigned), st);
-  unsigned arrived = 0;
+  unsigned arrived = withhold ? 1 : 0;
   const int64_t end = k + count;
   while (k < end && e == cudaSuccess) {
     const bool sp = special(k);
     int64_t to = k;
     unsigned barriers = 0;
-    while (to < end && special(to) == sp) {
+    while (to < end && to - k < kResidentIters && special(to) == sp) {
       barriers += sp ? (check(to) ? 4u : 3u) : 2u;
       ++to;
     }
@@ -1106,10 +1114,6 @@ static cudaError_t launch_flat(DeviceState* d, const IterArgs<P, S>& args, int* 
   }
   return e;
 }
-
-// Most iterations of one group of resident launches (whole chunks of k_check): the host looks
-// at the result, and other work gets the GPU, at least this often.
-constexpr int64_t kResidentIters = 1000;
 
 template <typename P, typename S>
 static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_result* res,
@@ -1202,6 +1206,7 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
   int verdict = STOP_NO;
   bool any = false;
   const bool resident = d->resident >= 0 && kt == nullptr;
+  const bool withhold_arrival = resident && g_withhold_arrival.exchange(0) != 0;
   if (resident) CK(cudaMemcpyAsync(&d->ctl->stop, &stop_state, sizeof(stop_state), cudaMemcpyHostToDevice, st));
   NvtxRange solve_range(d->precision == MCF_FP64 ? "pdmcf solve fp64"
                         : d->precision == MCF_BF16_F ? "pdmcf solve bf16" : "pdmcf solve fp32");
@@ -1212,7 +1217,8 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
     if (resident) {
       // the device evaluates the stop test: several chunks per launch, one with a check log
       if (!log) chunk = std::min<int64_t>((int64_t)kc * std::max<int64_t>(1, kResidentIters / kc), max_iters - k);
-      CK((launch_resident<P, S>(d, args, parity, k, chunk, max_iters, kc, o->k_adapt, stop, st)));
+      CK((launch_resident<P, S>(d, args, parity, k, chunk, max_iters, kc, o->k_adapt, stop,
+                                 withhold_arrival && k == 0, st)));
       CK(cudaMemcpyAsync(&stop_state, &d->ctl->stop, sizeof(stop_state), cudaMemcpyDeviceToHost, st));
     } else if (d->grid_flat > 0 && kt == nullptr) {
       CK((launch_flat<P, S>(d, args, &parity, k, chunk, max_iters, kc, o->k_adapt, st)));
@@ -1347,6 +1353,11 @@ static int copy_outputs_t(mcf_problem* p, DeviceState* d, mcf_result* res, cudaS
 
 extern "C" int mcf_test_withhold_next_copy(void) {
   pdmcf::g_withhold_request.store(1);
+  return MCF_OK;
+}
+
+extern "C" int mcf_test_withhold_next_arrival(void) {
+  pdmcf::g_withhold_arrival.store(1);
   return MCF_OK;
 }
 
