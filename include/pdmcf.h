@@ -99,9 +99,11 @@ typedef struct mcf_options {
                                 instances of that size (default 1)                         */
   int     shape;             /* kernel launch shape index (-1 = automatic); see
                                 mcf_shape_info. Lets tests and the tuner pick any shape
-                                whose capacity covers the problem. A shape named here runs
-                                one launch per phase; -1 may run the resident iteration
-                                (rows of up to 1024 entries) or the flat node phase        */
+                                whose capacity covers the problem. -1 may run the resident
+                                iteration (rows of up to 1024 entries) or the flat node
+                                phase, and so does the index of the shape that it stands for
+                                (mcf_kernel_times.shape of a timed solve with -1); any other
+                                shape runs one launch per phase                            */
   double  adapt_guard;       /* g: stop adapting omega (keep it constant, Sec. 2.4) from
                                 the iteration after a stop test where omega is more than a
                                 factor g^2 away from its value at the first stop test with
@@ -332,10 +334,12 @@ int mcf_project_capped_simplex_noalloc(int32_t n, int32_t m, int32_t ld, const f
                                        void* stream);
 
 /* Time every launch shape that covers this problem (register shapes up to 4x the smallest
- * sufficient capacity, and kinds 1 and 2 when opts->precision is not MCF_FP64) with
- * 3 + 10 iterations each, and return the fastest in *best_shape (for mcf_options.shape) and
- * its time per iteration in *ms_per_iter (may be NULL). Uses the problem's device state; the
- * next solve of the problem starts cold. */
+ * sufficient capacity, and kinds 1 and 2 when opts->precision is not MCF_FP64) with warm solves of
+ * 10 iterations each (100 where those take under 2 ms) as mcf_solve runs them, and return the
+ * fastest in *best_shape (for mcf_options.shape) and its time per iteration in *ms_per_iter (may
+ * be NULL), the call included. The shape that the automatic choice stands for is among them, with
+ * the kernels of the automatic choice. Uses the problem's device state; the next solve of the
+ * problem starts cold. */
 int mcf_autotune(mcf_problem* p, const mcf_options* opts, int* best_shape, double* ms_per_iter);
 
 /* Launch shape table: shape s gives `group` threads per edge/node, each holding `vpt`

@@ -1,0 +1,50 @@
+"""mcf_autotune returns a shape that is not slower than the automatic choice, also where that choice
+runs the resident iteration or the flat node phase, and naming the shape that the automatic choice
+stands for runs the same kernels. A shape that launched the per-phase kernels instead took 2.8
+times as long at n = 100 and 13 times as long with an exponent for each pair in FP64; the bound of
+1.5 leaves room for the clock."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2501_17996_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _powij(n, seed):
+    inst = I.ring_random_instance(n, 9, seed, "u1_10", "pow", gamma=0.5)
+    inst.gamma = np.random.default_rng(seed).uniform(0.3, 0.7, size=(n, n))
+    return inst
+
+
+def _seconds(p, **opts):
+    p.solve(want_T=False, stop_mode="none", max_iters=200, **opts)
+    best = 1e9
+    for _ in range(5):
+        t0 = time.perf_counter()
+        p.solve(want_T=False, stop_mode="none", max_iters=200, warm_start=1, **opts)
+        best = min(best, time.perf_counter() - t0)
+    return best
+
+
+@pytest.mark.parametrize("make,precision", [
+    (lambda: I.mid(0), "fp32"), (lambda: _powij(203, 1), "fp64"),
+    (lambda: I.ring_random_instance(2500, 8, 2, "u1_10", "log"), "fp32")])
+def test_tuned_shape_is_not_slower_than_the_automatic_one(lib, make, precision):
+    with lib.Problem(make()) as p:
+        shape, ms = p.autotune(precision=precision, stop_mode="none")
+        assert ms > 0
+        auto = _seconds(p, precision=precision)
+        assert _seconds(p, precision=precision, shape=shape) <= 1.5 * auto
+
+
+@pytest.mark.parametrize("n,precision", [(100, "fp32"), (203, "fp64"), (2500, "fp32")])
+def test_the_automatic_choice_by_its_name(lib, n, precision):
+    opts = dict(precision=precision, stop_mode="none", max_iters=23, k_check=10)
+    with lib.Problem(I.ring_random_instance(n, 4, 3, "lognormal", "pow", gamma=0.4)) as p:
+        r, _ = p.solve_timed(**opts)
+        a = p.solve(want_T=True, **opts)
+        b = p.solve(want_T=True, shape=r["shape"], **opts)
+    assert np.array_equal(a["T"], b["T"]) and a["omega"] == b["omega"]
