@@ -125,15 +125,20 @@ __device__ __forceinline__ float prox_pow_start(float y, float k, float c1) {
   return t;
 }
 
+// How far off the start of prox_pow_traffic may be, times c1 + 1. What the correction leaves grows as
+// ((c1 + 1) d)^4 for two steps (FP64: at most 8.6e-17 of the root and 1.0e-16 of the traffic at the
+// limit, exponents 0.05 to 0.95) and as ((c1 + 1) d)^2 for one (FP32: 4e-8): below half a last place.
+template <typename P> __device__ constexpr P prox_reach() { return sizeof(P) == 8 ? P(1e-4) : P(2e-4); }
+
 // prox of the power utility and the traffic t = T(Y^) = (w gamma / -Y^)^(1/(1-gamma)) of its
 // result, given wg = (w gamma)^(1/(1-gamma)). With c1 + 1 = 1/(1-gamma) the root equation of
 // prox_pow is t^(c1+1) (t + y) = beta wg (its constant c1 (1/gamma - 1) is 1), and the traffic
 // is wg / t^(c1+1). One full-precision power serves the whole search: the FP32 start is good to
 // about 1e-5, one Newton step leaves the square of that, and for the second the power at the
-// moved point follows from the binomial series (1 + d)^c1, whose fourth-order rest is below
-// the last place. (The search of prox_pow takes about eight powers, each some hundred FP64
-// instructions on a unit that runs at 1/64 of FP32.) A start that turns out farther off, or
-// out of FP32's range, takes the full search.
+// moved point follows from the binomial series (1 + d)^c1 up to its third order. (The search of
+// prox_pow takes about eight powers, each some hundred FP64 instructions on a unit that runs at
+// 1/64 of FP32.) A start that turns out farther off than prox_reach, or out of FP32's range, takes
+// the full search.
 template <typename P>
 __device__ __forceinline__ P prox_pow_traffic(P y, P beta, P w, P wg, P gamma, P& traffic) {
   if (gamma == P(0.5)) {
@@ -151,7 +156,7 @@ __device__ __forceinline__ P prox_pow_traffic(P y, P beta, P w, P wg, P gamma, P
     const P a = c1 + P(2), b = (c1 + P(1)) * y;
     const P t1 = fmax(t0 - (p0 * t0 * (t0 + y) - k) / (p0 * (a * t0 + b)), tlo);
     const P d = (t1 - t0) / t0;
-    if (fabs(d) < P(1e-3)) {
+    if (fabs(d) * (c1 + P(1)) < prox_reach<P>()) {
       const P p1 = p0 * (P(1) + c1 * d * (P(1) + (c1 - P(1)) * P(0.5) * d *
                                                    (P(1) + (c1 - P(2)) * P(1.0 / 3.0) * d)));
       P t = t1, p = p1;
