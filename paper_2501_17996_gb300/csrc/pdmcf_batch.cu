@@ -108,15 +108,11 @@ int batch_admit_shape(const mcf_problem* p) {
 
 static int node_pieces_per(int n) { return batch_pieces_per((n + 7) / 8 * 8); }
 
-// What admission counts for the sums: one set per edge and per node, whatever the pieces per node
-// (they add about 1 % of the state at most), so that a budget admits the same requests for any BATCH_N.
+// The slot's sums, as they are allocated and as admission counts them: one set per edge and per piece
+// (the pieces of a node's column add up to 1 % of the state).
 int64_t BatchEngine::extra_bytes(const mcf_problem* p) {
-  return (int64_t)sizeof(double) * ((int64_t)p->m * (1 + CHECK_PARTS) + (int64_t)p->n * NODE_PARTS);
-}
-
-static size_t parts_bytes(const mcf_problem* p) {
-  return sizeof(double) * ((size_t)p->m * (1 + CHECK_PARTS) +
-                           (size_t)p->n * node_pieces_per(p->n) * NODE_PARTS);
+  return (int64_t)sizeof(double) * ((int64_t)p->m * (1 + CHECK_PARTS) +
+                                    (int64_t)p->n * node_pieces_per(p->n) * NODE_PARTS);
 }
 
 BatchEngine::BatchEngine(int device, int max_slots)
@@ -218,7 +214,7 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   if (rc != MCF_OK) return rc;
   BatchSlot& sl = slots_[s];
   sl = BatchSlot();
-  sl.parts = alloc_parts(parts_bytes(p));
+  sl.parts = alloc_parts((size_t)extra_bytes(p));
   if (!sl.parts) {
     cudaStreamSynchronize(stream_);   // the state's preparation
     sl = BatchSlot();
@@ -276,7 +272,7 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   hs.stall_frozen = 0;
   lists_dirty_ = true;
   // read before the next chunk's copy back writes the mirror: same stream
-  BCK(cudaMemsetAsync(sl.parts, 0, parts_bytes(p), stream_));
+  BCK(cudaMemsetAsync(sl.parts, 0, (size_t)extra_bytes(p), stream_));
   BCK(cudaMemcpyAsync(d_insts_ + s, &h_insts_[s], sizeof(bi), cudaMemcpyHostToDevice, stream_));
   BCK(cudaMemcpyAsync(d_sc_ + s, &hs, sizeof(hs), cudaMemcpyHostToDevice, stream_));
   (void)warm;

@@ -63,7 +63,7 @@ class BatchEngine {
   // on other streams once the engine's has been waited for: by this call or a later one with wait.
   void release(int slot, bool wait = true);
   const BatchSlot& slot(int s) const { return slots_[s]; }
-  static int64_t extra_bytes(const mcf_problem* p);   // engine buffers per instance, as admission counts them
+  static int64_t extra_bytes(const mcf_problem* p);   // engine buffers per instance
 
  private:
   double* alloc_parts(size_t bytes);
