@@ -25,6 +25,7 @@ namespace pdmcf {
 
 // Solver-side helpers (pdmcf_solver.cu).
 cudaMemPool_t state_pool(int device);
+cudaError_t pool_alloc(void** p, size_t bytes, cudaMemPool_t pool, cudaStream_t st);
 int batch_prepare_state(mcf_problem* p, const mcf_options* o, cudaStream_t st, bool* warm);
 void batch_state_pointers(mcf_problem* p, BatchInst* bi, int* parity);
 void batch_finish_state(mcf_problem* p, int parity, const DevScalars& s, cudaStream_t st);
@@ -428,18 +429,7 @@ std::vector<int> BatchEngine::take_finished() {
 // batch of 64 small networks took 6.2 ms around one iteration, now 3.8.
 double* BatchEngine::alloc_parts(size_t bytes) {
   double* ptr = nullptr;
-  cudaError_t e;
-  if (pool_) {
-    e = cudaMallocFromPoolAsync((void**)&ptr, bytes, pool_, stream_);
-    if (e == cudaErrorMemoryAllocation) {   // return the pool's cached memory and retry
-      cudaGetLastError();
-      cudaStreamSynchronize(stream_);
-      cudaMemPoolTrimTo(pool_, 0);
-      e = cudaMallocFromPoolAsync((void**)&ptr, bytes, pool_, stream_);
-    }
-  } else {
-    e = cudaMalloc((void**)&ptr, bytes);
-  }
+  const cudaError_t e = pool_ ? pool_alloc((void**)&ptr, bytes, pool_, stream_) : cudaMalloc((void**)&ptr, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return nullptr;

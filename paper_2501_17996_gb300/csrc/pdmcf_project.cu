@@ -17,7 +17,9 @@
 
 namespace pdmcf {
 
-cudaMemPool_t state_pool(int device);   // pdmcf_solver.cu
+// pdmcf_solver.cu
+cudaMemPool_t state_pool(int device);
+cudaError_t pool_alloc(void** p, size_t bytes, cudaMemPool_t pool, cudaStream_t st);
 
 // Fixed-order sum of x[0..count) into *out by one block of 1024 threads: thread t adds x[t],
 // x[t + 1024], ... (coalesced; a segment per thread took 20 us at 30 000 columns), then a tree.
@@ -362,8 +364,7 @@ extern "C" int mcf_project_capped_simplex(int32_t n, int32_t m, int32_t ld, cons
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) pool = state_pool(dev);
     const size_t bytes = ((size_t)m + 1) * sizeof(double);
-    const cudaError_t ea = pool ? cudaMallocFromPoolAsync((void**)&scratch, bytes, pool, st)
-                                : cudaMalloc((void**)&scratch, bytes);
+    const cudaError_t ea = pool ? pool_alloc((void**)&scratch, bytes, pool, st) : cudaMalloc((void**)&scratch, bytes);
     if (ea != cudaSuccess) {
       cudaGetLastError();
       set_error("device allocation of the projection scratch failed");

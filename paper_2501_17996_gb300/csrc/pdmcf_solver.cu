@@ -208,8 +208,15 @@ cudaMemPool_t state_pool(int device) {
   std::lock_guard<std::mutex> g(g_pool_mu);
   PoolSlot& s = g_pools[device];
   if (s.unsupported) return nullptr;
-  const unsigned long long ctx = current_context_id();
-  if (s.pool && (ctx == 0 || ctx == s.ctx)) return s.pool;
+  unsigned long long ctx = current_context_id();
+  if (ctx == 0) {   // a thread that has not used the device yet has no context current: bring it up
+    if (cudaSetDevice(device) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    ctx = current_context_id();
+  }
+  if (s.pool && (ctx == 0 || ctx == s.ctx)) return s.pool;   // (0: contexts have no ids here)
   int ok = 0;
   if (cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, device) != cudaSuccess || !ok) {
     cudaGetLastError();
@@ -233,6 +240,19 @@ cudaMemPool_t state_pool(int device) {
   return pool;
 }
 
+// `bytes` from the pool in st's order; where there are none left, once more after the pool's cached
+// memory has been given back.
+cudaError_t pool_alloc(void** p, size_t bytes, cudaMemPool_t pool, cudaStream_t st) {
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaStreamSynchronize(st);
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
+  return e;
+}
+
 // The kernels' vector loads and bulk copies need 16-byte aligned buffers (cudaMalloc returns
 // 256-byte aligned ones); a buffer that is not aligned is refused rather than used.
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -250,13 +270,7 @@ static bool dalloc(DeviceState* d, void** p, size_t bytes) {
   *p = nullptr;
   cudaError_t e;
   if (d->pool) {
-    e = cudaMallocFromPoolAsync(p, bytes, d->pool, d->own_stream);
-    if (e == cudaErrorMemoryAllocation) {   // return the pool's cached memory and retry
-      cudaGetLastError();
-      cudaStreamSynchronize(d->own_stream);
-      cudaMemPoolTrimTo(d->pool, 0);
-      e = cudaMallocFromPoolAsync(p, bytes, d->pool, d->own_stream);
-    }
+    e = pool_alloc(p, bytes, d->pool, d->own_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(d->own_stream);
   } else {
     e = cudaMalloc(p, bytes);
