@@ -177,9 +177,9 @@ __device__ __forceinline__ void batch_edges(const BatchInst& I, int e, int e1) {
         q[v][u + 1] = ci < nchunks ? qq.y : floor;
       }
     }
-    GroupScratch<32>* none = nullptr;   // warp groups reduce without scratch memory
+    GroupScratch<32> none;   // warp groups reduce without scratch memory
     int phase = 0;
-    const float mu = project_mu<32, V, VW, float>(q, mc, 0.f, floor, *none, phase);
+    const float mu = project_mu<32, V, VW, float>(q, mc, 0.f, floor, none, phase);
     float dloc = 0.f;
     float* fn = F1 + (size_t)e * ld;
 #pragma unroll

@@ -636,9 +636,9 @@ __device__ __forceinline__ P edge_phase(const IterArgs<P, S>& a, int par, P alph
     if constexpr (std::is_same<P, double>::value) {
       mu = project_mu64<VPT, VW>(q, cap, floor);
     } else {
-      GroupScratch<32>* none = nullptr;   // warp groups reduce without scratch memory
+      GroupScratch<32> none;   // warp groups reduce without scratch memory
       int phase = 0;
-      mu = project_mu<32, VPT, VW, P>(q, cap, P(0), floor, *none, phase);
+      mu = project_mu<32, VPT, VW, P>(q, cap, P(0), floor, none, phase);
     }
     P dloc = P(0);
 #pragma unroll
