@@ -209,6 +209,10 @@ struct NodeItem {
   P po[N], yo[N], yl[N];
 };
 
+// The utility; BF16-stored F comes here with log utility only (setup_resident, setup_flat).
+template <typename P, typename S>
+__device__ __forceinline__ int node_kind(const IterArgs<P, S>& a) { return sizeof(S) == 2 ? 0 : a.kind; }
+
 template <typename P, typename S, int N>
 __device__ __forceinline__ void node_data(const IterArgs<P, S>& a, const NodePiece& q, NodeItem<P, N>& x) {
   if (q.c * N >= a.ld) return;
@@ -219,7 +223,7 @@ __device__ __forceinline__ void node_data(const IterArgs<P, S>& a, const NodePie
 #pragma unroll
     for (int u = 0; u < N; ++u) x.gv[u] = a.gamma;
   }
-  if (a.kind == 1 && sizeof(S) != 2) {
+  if (node_kind(a) == 1) {
 #pragma unroll
     for (int u = 0; u < N; ++u)
       x.wg[u] = x.gv[u] == P(0.5) ? P(0) : pow(x.wv[u] * x.gv[u], P(1) / (P(1) - x.gv[u]));
@@ -301,6 +305,7 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
   const int j = q.j, c = q.c;
   const P rho = a.rho, inv_rho = P(1) / rho;
   const size_t o = (size_t)j * a.ld + (size_t)c * N;
+  const int kind = node_kind(a);
   P yn[N], th_v[N], up_v[N], yh_v[N];
 #pragma unroll
   for (int u = 0; u < N; ++u) {
@@ -312,8 +317,7 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
     P delta, tr = P(0);
     if (live) {
       const P vv = x.yo[u] + (x.yl[u] - beta * fplus_at);
-      // (BF16-stored F: node_kernel's search, see setup_resident)
-      if (a.kind == 0 || sizeof(S) == 2) tr = prox_traffic<P>(a.kind, vv, beta, x.wv[u], x.gv[u]);
+      if (kind == 0) tr = prox_traffic<P>(0, vv, beta, x.wv[u], x.gv[u]);
       else prox_pow_traffic<P>(vv, beta, x.wv[u], x.wg[u], x.gv[u], tr);
       delta = -beta * (fplus_at + tr);
     } else {
@@ -334,11 +338,11 @@ __device__ __forceinline__ void node_update(const IterArgs<P, S>& a, int par, co
       if (live) {
         if (!(th > P(0))) loc[1] += P(1);
         else {
-          loc[2] += util_value<P>(a.kind, th, x.wv[u], x.gv[u]);
-          up_v[u] = util_grad<P>(a.kind, th, x.wv[u], x.gv[u]);
+          loc[2] += util_value<P>(kind, th, x.wv[u], x.gv[u]);
+          up_v[u] = util_grad<P>(kind, th, x.wv[u], x.gv[u]);
         }
         if (yhat < P(0)) {
-          loc[3] += util_conj_neg<P>(a.kind, yhat, x.wv[u], x.gv[u]);
+          loc[3] += util_conj_neg<P>(kind, yhat, x.wv[u], x.gv[u]);
           const P dt = tr - th;
           loc[4] = fma(dt, dt, loc[4]);
         } else {
