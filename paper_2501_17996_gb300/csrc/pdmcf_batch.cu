@@ -32,17 +32,49 @@ void batch_finish_state(mcf_problem* p, int parity, const DevScalars& s, cudaStr
 
 // ------------------------------------------------------------------ scalar kernel
 
+constexpr int SCALAR_BLOCK = 512;
+
 struct BatchScalarArgs {
   const BatchInst* insts;
   const int* slots;
   const int* nslots;
 };
 
-// One block per resident instance: fixed-order FP64 sums of its per-edge and per-node
+// Sums of K consecutive fields over nb items of `stride` doubles by the block's threads, in a
+// fixed order; thread 0 gets them. Thread t adds items t, t + 512, ..., all K fields of an item at
+// once, several items in flight. (A contiguous segment per thread, field by field, took most of the
+// 95 us of this kernel at a stop test of n = 3000, m = 24 000.)
+template <int K>
+__device__ __forceinline__ void block_sums(const double* __restrict__ base, int nb, size_t stride, double* out,
+                                           double (&sh)[8][SCALAR_BLOCK / 32]) {
+  constexpr int W = K > 4 ? 8 : K > 1 ? 4 : 1;   // warp_sums takes a power of two
+  double s[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) s[k] = 0.0;
+#pragma unroll 8
+  for (int b = threadIdx.x; b < nb; b += SCALAR_BLOCK)
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k] += base[(size_t)b * stride + k];
+  const double sum = warp_sums<W>(s);
+  const int lane = threadIdx.x & 31, field = lane / (32 / W);
+  if (lane % (32 / W) == 0) sh[field][threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double t = 0.0;
+      for (int w = 0; w < SCALAR_BLOCK / 32; ++w) t += sh[k][w];
+      out[k] = t;
+    }
+  }
+  __syncthreads();
+}
+
+// One block per resident instance: fixed-order FP64 sums of its per-edge and per-piece
 // parts, the shared scalar update, parity flip and the stop rule (Algorithm 2.1, step 1,
 // evaluated on the instance's own check iterations).
-__global__ void __launch_bounds__(256) batch_scalar_kernel(BatchScalarArgs a) {
-  __shared__ double sh[256];
+__global__ void __launch_bounds__(SCALAR_BLOCK) batch_scalar_kernel(BatchScalarArgs a) {
+  __shared__ double sh[8][SCALAR_BLOCK / 32];
   if ((int)blockIdx.x >= *a.nslots) return;
   const BatchInst& I = a.insts[a.slots[blockIdx.x]];
   BatchScalars* bs = I.sc;
@@ -63,15 +95,15 @@ __global__ void __launch_bounds__(256) batch_scalar_kernel(BatchScalarArgs a) {
     }
     return;
   }
-  const int np = I.n * I.per;
-  const double dF2 = det_sum(I.pe, I.m, 1, 0, sh);
-  const double dY2 = det_sum(I.pn, np, NODE_PARTS, 0, sh);
-  double nodep[NODE_PARTS];
-  double chk[CHECK_PARTS];
-  if (check) {
-    for (int f = 1; f < NODE_PARTS; ++f) nodep[f] = det_sum(I.pn, np, NODE_PARTS, f, sh);
-    for (int f = 0; f < CHECK_PARTS; ++f) chk[f] = det_sum(I.pc, I.m, CHECK_PARTS, f, sh);
+  double dF2, nodep[NODE_PARTS], chk[CHECK_PARTS];
+  block_sums<1>(I.pe, I.m, 1, &dF2, sh);
+  if (check) {   // after a check phase a node's pieces are in its first one
+    block_sums<NODE_PARTS>(I.pn, I.n, (size_t)I.per * NODE_PARTS, nodep, sh);
+    block_sums<CHECK_PARTS>(I.pc, I.m, CHECK_PARTS, chk, sh);
+  } else {
+    block_sums<1>(I.pn, I.n * I.per, NODE_PARTS, nodep, sh);
   }
+  const double dY2 = nodep[0];
   if (threadIdx.x != 0) return;
   DevScalars* s = &bs->s;
   scalar_update(s, dF2, dY2, nodep, chk, check);
@@ -330,7 +362,7 @@ int BatchEngine::launch_iteration(cudaStream_t st, bool with_check) {
   BCK(launch(with_check ? T.node_chk : T.node, NUM_GROUPS, with_check ? grid_node_chk_ : grid_node_, 256));
   if (with_check) BCK(launch(T.check, NUM_GROUPS, grid_check_, 256));
   BatchScalarArgs sa{d_insts_, d_slot_list_, d_nslots_};
-  batch_scalar_kernel<<<max_slots_, 256, 0, st>>>(sa);
+  batch_scalar_kernel<<<max_slots_, SCALAR_BLOCK, 0, st>>>(sa);
   BCK(cudaGetLastError());
   return MCF_OK;
 }
