@@ -459,7 +459,7 @@ __device__ __forceinline__ void check_phase(const IterArgs<P, S>& a, int par, P 
 
 // ------------------------------------------------------------------ scalar tail
 
-// Scalar tail in block 0: a warp per field sums the CTAs' FP64 partials in a fixed order, then
+// Scalar tail in block 0: a warp per field sums the shares' FP64 partials in a fixed order, then
 // one thread updates the scalars and evaluates the stop test.
 template <typename P, typename S, int BLOCK>
 __device__ __forceinline__ void scalar_phase(const IterArgs<P, S>& a, const ResidentArgs& ra, long long k,
@@ -473,7 +473,7 @@ __device__ __forceinline__ void scalar_phase(const IterArgs<P, S>& a, const Resi
                                               : a.part_check + (f - 1 - NODE_PARTS);
     const int stride = f == 0 ? 1 : f <= NODE_PARTS ? NODE_PARTS : CHECK_PARTS;
     double s = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(base + (size_t)b * stride);
+    for (int b = lane; b < ra.ctas; b += 32) s += __ldcg(base + (size_t)b * stride);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) field[f] = s;
@@ -692,20 +692,21 @@ __device__ __forceinline__ P edge_phase(const IterArgs<P, S>& a, int par, P alph
 
 // ------------------------------------------------------------------ the kernels
 
-struct ResidentPlace {   // this warp's share of the work
+// The work of a phase is dealt to `ctas` CTAs; this warp's part as one of CTA `cta`.
+struct ResidentPlace {
   int e0, e1, warp, nwarps;
   unsigned pieces;   // of the node phase: this warp takes warp, warp + nwarps, ...
 };
 
 template <int NW>
-__device__ __forceinline__ ResidentPlace resident_place(int n, int m, int ld, int N) {
+__device__ __forceinline__ ResidentPlace resident_place(int n, int m, int ld, int N, int cta, int ctas) {
   ResidentPlace w;
   // numbered across the CTAs first, so that few pieces spread over all SMs
-  w.warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  w.nwarps = gridDim.x * NW;
+  w.warp = (threadIdx.x >> 5) * ctas + cta;
+  w.nwarps = ctas * NW;
   // consecutive edges per CTA (their heads' dual rows are shared in L1)
-  w.e0 = (int)((long long)m * blockIdx.x / gridDim.x) + (threadIdx.x >> 5);
-  w.e1 = (int)((long long)m * (blockIdx.x + 1) / gridDim.x);
+  w.e0 = (int)((long long)m * cta / ctas) + (threadIdx.x >> 5);
+  w.e1 = (int)((long long)m * (cta + 1) / ctas);
   w.pieces = (unsigned)n * ((unsigned)(ld + 32 * N - 1) / (32 * N));
   return w;
 }
@@ -726,7 +727,7 @@ resident_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant_
   constexpr int NW = BLOCK / 32;
   __shared__ int failed;
   if (__ldcg(&ra.ctl->stop.verdict) != STOP_NO) return;
-  const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N);
+  const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N, blockIdx.x, gridDim.x);
   const P alpha = (P)__ldcg(&a.sc->alpha), beta = (P)__ldcg(&a.sc->beta);
   NodePiece piece;
   NodeItem<P, N> x;      // data of the first piece: stays in registers when it is the only one
@@ -764,14 +765,16 @@ resident_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant_
   }
 }
 
-// Iterations with a scalar tail (a multiple of k_adapt, or a stop test), usually one or two.
+// Iterations with a scalar tail (a multiple of k_adapt, or a stop test), usually one or two. The work
+// is split into the shares of ra.ctas CTAs whatever the grid: CTA b of a smaller one takes the shares b,
+// b + gridDim.x, ... one after the other. So the sums, and with them the iterates, do not depend on
+// the grid, and solves under way at the same time can run on a part of the SMs each (ResidentTurn).
 template <typename P, typename S, int VPT, int N, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1)
 resident_special_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_constant__ ResidentArgs ra) {
   constexpr int NW = BLOCK / 32;
   __shared__ int failed;
   if (__ldcg(&ra.ctl->stop.verdict) != STOP_NO) return;
-  const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N);
   resident_start(a, failed);
   __syncthreads();
   if (failed) return;
@@ -782,32 +785,45 @@ resident_special_kernel(const __grid_constant__ IterArgs<P, S> a, const __grid_c
     const long long k = ra.k + i;
     const bool check = (k + 1) % ra.k_check == 0 || k + 1 >= ra.max_iters;
     const P alpha = (P)__ldcg(&a.sc->alpha), beta = (P)__ldcg(&a.sc->beta);
-    bool ok;
-    const P dsum = edge_phase<P, S, VPT, NW>(a, par, alpha, w.e0, w.e1, bar, false, ok);
+#pragma unroll 1
+    for (int share = blockIdx.x; share < ra.ctas; share += gridDim.x) {
+      const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N, share, ra.ctas);
+      bool ok;
+      double v1[1] = {(double)edge_phase<P, S, VPT, NW>(a, par, alpha, w.e0, w.e1, bar, false, ok)};
+      block_sum_write<BLOCK, 1>(v1, a.part_edge + share);
+      __syncthreads();   // its scratch is used again
+    }
     bar.arrive();
     if (!bar.wait()) return;
-    double acc[NODE_PARTS];
+#pragma unroll 1
+    for (int share = blockIdx.x; share < ra.ctas; share += gridDim.x) {
+      const ResidentPlace w = resident_place<NW>(a.n, a.m, a.ld, N, share, ra.ctas);
+      double acc[NODE_PARTS];
 #pragma unroll
-    for (int q = 0; q < NODE_PARTS; ++q) acc[q] = 0.0;
-    NodePiece piece;
-    NodeItem<P, N> x;
-    if ((unsigned)w.warp < w.pieces) {
-      node_place<P, S, N>(a, w.warp, piece);
-      piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
-      node_data<P, S, N>(a, piece, x);
-      node_state<P, S, N>(a, par, piece, x);
+      for (int q = 0; q < NODE_PARTS; ++q) acc[q] = 0.0;
+      NodePiece piece;
+      NodeItem<P, N> x;
+      if ((unsigned)w.warp < w.pieces) {
+        node_place<P, S, N>(a, w.warp, piece);
+        piece.edge = node_edge(a, piece, (int)(threadIdx.x & 31));
+        node_data<P, S, N>(a, piece, x);
+        node_state<P, S, N>(a, par, piece, x);
+      }
+      if (check) node_pieces<P, S, N, true>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
+      else node_pieces<P, S, N, false>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
+      block_sum_write<BLOCK, NODE_PARTS>(acc, a.part_node + (size_t)share * NODE_PARTS);
+      __syncthreads();
     }
-    if (check) node_pieces<P, S, N, true>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
-    else node_pieces<P, S, N, false>(a, par, w.warp, w.pieces, w.nwarps, piece, x, beta, acc);
-    double v1[1] = {(double)dsum};
-    block_sum_write<BLOCK, 1>(v1, a.part_edge + blockIdx.x);
-    block_sum_write<BLOCK, NODE_PARTS>(acc, a.part_node + (size_t)blockIdx.x * NODE_PARTS);
     bar.arrive();
     if (!bar.wait()) return;
     if (check) {
-      double cacc[CHECK_PARTS];
-      check_phase<P, S>(a, par, alpha, w.warp, w.nwarps, cacc);
-      block_sum_write<BLOCK, CHECK_PARTS>(cacc, a.part_check + (size_t)blockIdx.x * CHECK_PARTS);
+#pragma unroll 1
+      for (int share = blockIdx.x; share < ra.ctas; share += gridDim.x) {
+        double cacc[CHECK_PARTS];
+        check_phase<P, S>(a, par, alpha, (threadIdx.x >> 5) * ra.ctas + share, ra.ctas * NW, cacc);
+        block_sum_write<BLOCK, CHECK_PARTS>(cacc, a.part_check + (size_t)share * CHECK_PARTS);
+        __syncthreads();
+      }
       bar.arrive();
       if (!bar.wait()) return;
     }

@@ -61,6 +61,7 @@ struct ResidentArgs {
   ResidentCtl* ctl;
   long long k;              // first iteration of this launch
   int count;                // iterations of this launch
+  int ctas;                 // shares of the work (the grid may be smaller)
   unsigned arrived;         // barrier arrivals of the group's earlier launches
   long long max_iters;      // of the solve; a check falls on multiples of k_check and on the last
   long long k_check;

@@ -16,6 +16,7 @@
 #include <cstring>
 #include <limits>
 #include <mutex>
+#include <optional>
 #include <string>
 #include <vector>
 
@@ -136,6 +137,7 @@ struct DeviceState {
   size_t tma_smem = 0;
   // resident iteration (resident >= 0): many iterations per cooperative launch
   int resident = -1, grid_resident = 0;
+  int half_resident = 0;   // grid while other resident solves are under way (0: the same, see ResidentTurn)
   ResidentCtl* ctl = nullptr;
   // iterations without a scalar tail where the resident iteration does not serve: the register
   // edge phase and the node phase over pieces (grid_flat > 0)
@@ -590,6 +592,8 @@ static int setup_resident(DeviceState* d, int want) {
   const int64_t warps = std::max<int64_t>(d->m, (int64_t)d->n * ((d->ld + 31) / 32));
   d->resident = t;
   d->grid_resident = (int)std::min<int64_t>(sms, (warps + 3) / 4);
+  const int half = sms / 2;
+  d->half_resident = d->grid_resident > half && warps <= (int64_t)half * (B / 32) ? half : 0;
   return MCF_OK;
 }
 
@@ -1075,6 +1079,29 @@ static void write_check_line(FILE* f, const DevScalars& h, int n, int m, int pre
 static std::atomic<int> g_withhold_request{0};
 static bool take_withhold_request() { return g_withhold_request.exchange(0) != 0; }
 
+// Resident solves under way on a device. A resident CTA fills an SM, so solves on several host threads
+// take turns where each takes all SMs. A network whose items fill the warps of half the SMs at most
+// loses little on one half, so while several are under way it runs on one and two run at a time (the
+// iterates do not depend on it, see resident_special_kernel). Networks with more work gain nothing that
+// way (n = 300: 9.3 us per iteration in turn, 10.0 at once; n = 1000: 47.2 and 47.7). Us per
+// iteration and solve with 1, 2, 4, 8 and 16 threads, a network of n = 100, m = 1000 each: 5.4, 3.3, 3.1,
+// 3.0, 3.0; all in turn 5.3; the per-phase kernels, whose launches overlap, 16.7, 9.0, 4.7, 2.5, 1.4.
+class ResidentTurn {
+ public:
+  explicit ResidentTurn(const DeviceState* d) : d_(d), under_way_(under_way(d->device)) { under_way_.fetch_add(1); }
+  ~ResidentTurn() { under_way_.fetch_sub(1); }
+  ResidentTurn(const ResidentTurn&) = delete;
+  int grid() const { return d_->half_resident > 0 && under_way_.load() > 1 ? d_->half_resident : d_->grid_resident; }
+
+ private:
+  static std::atomic<int>& under_way(int device) {
+    static std::atomic<int> n[kPoolDevices];
+    return n[device % kPoolDevices];
+  }
+  const DeviceState* d_;
+  std::atomic<int>& under_way_;
+};
+
 // mcf_test_withhold_next_arrival: one pending request, taken by the next resident solve.
 static std::atomic<int> g_withhold_arrival{0};
 
@@ -1089,7 +1116,7 @@ constexpr int64_t kResidentIters = 1000;
 template <typename P, typename S>
 static cudaError_t launch_resident(DeviceState* d, const IterArgs<P, S>& args, int parity, int64_t k, int64_t count,
                                    int64_t max_iters, int64_t kc, int64_t k_adapt, const StopRule& rule,
-                                   bool withhold, cudaStream_t st) {
+                                   int grid, bool withhold, cudaStream_t st) {
   const ResidentTable<P, S>& T = get_resident<P, S>();
   k_adapt = std::max<int64_t>(1, k_adapt);
   auto check = [&](int64_t i) { return (i + 1) % kc == 0 || i + 1 >= max_iters; };
@@ -1108,11 +1135,11 @@ static cudaError_t launch_resident(DeviceState* d, const IterArgs<P, S>& args, i
     --barriers;   // the end of the kernel is the last one
     IterArgs<P, S> a = args;
     a.parity = parity;
-    ResidentArgs ra{d->ctl, k, (int)(to - k), arrived, max_iters, kc, rule};
+    ResidentArgs ra{d->ctl, k, (int)(to - k), d->grid_resident, arrived, max_iters, kc, rule};
     void* kargs[] = {&a, &ra};
     e = cudaLaunchCooperativeKernel(sp ? (const void*)T.special[d->resident] : (const void*)T.plain[d->resident],
-                                    dim3(d->grid_resident), dim3(RESIDENT_BLOCK), kargs, 0, st);
-    arrived += barriers * (unsigned)d->grid_resident;
+                                    dim3(grid), dim3(RESIDENT_BLOCK), kargs, 0, st);
+    arrived += barriers * (unsigned)grid;
     if ((to - k) & 1) parity ^= 1;
     k = to;
   }
@@ -1234,6 +1261,8 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
   int verdict = STOP_NO;
   bool any = false;
   const bool resident = d->resident >= 0 && kt == nullptr;
+  std::optional<ResidentTurn> turn;
+  if (resident) turn.emplace(d);
   const bool withhold_arrival = resident && g_withhold_arrival.exchange(0) != 0;
   if (resident) CK(cudaMemcpyAsync(&d->ctl->stop, &stop_state, sizeof(stop_state), cudaMemcpyHostToDevice, st));
   NvtxRange solve_range(d->precision == MCF_FP64 ? "pdmcf solve fp64"
@@ -1246,7 +1275,7 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
       // the device evaluates the stop test: several chunks per launch, one with a check log
       if (!log) chunk = std::min<int64_t>((int64_t)kc * std::max<int64_t>(1, kResidentIters / kc), max_iters - k);
       CK((launch_resident<P, S>(d, args, parity, k, chunk, max_iters, kc, o->k_adapt, stop,
-                                 withhold_arrival && k == 0, st)));
+                                 turn->grid(), withhold_arrival && k == 0, st)));
       CK(cudaMemcpyAsync(&stop_state, &d->ctl->stop, sizeof(stop_state), cudaMemcpyDeviceToHost, st));
     } else if (d->grid_flat > 0 && kt == nullptr) {
       CK((launch_flat<P, S>(d, args, &parity, k, chunk, max_iters, kc, o->k_adapt, st)));
@@ -1288,6 +1317,7 @@ static int solve_t(mcf_problem* p, DeviceState* d, const mcf_options* o, mcf_res
     }
     verdict = resident ? stop_state.verdict : stop_test(h, stop, stop_state);
   }
+  turn.reset();
   int status = o->stop_mode == MCF_STOP_NONE ? MCF_OK : MCF_ERR_NOT_CONVERGED;
   if (verdict == STOP_CONVERGED) status = MCF_OK;
   if (verdict == STOP_NUMERIC) {
