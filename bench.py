@@ -7,7 +7,11 @@ iteration (edge phase, node phase, scalar tail; every k_check-th iteration also 
 residual check), launched through the C ABI on torch's current stream.
 
 Printed JSON line (rank 0):
-  value     iterations/s of the whole job (sum over ranks / max time), inputs resident in HBM
+  value     iterations/s of the whole job (sum over ranks / max time), inputs resident in HBM,
+            by the launches that mcf_solve_timed puts events around (one per phase)
+  solve     the same number of iterations by one plain mcf_solve on this rank, whose automatic
+            kernels are others on shorter rows (the resident iteration, the flat node phase);
+            on the default workload they are the same launches
   e2e       the same metric through the public API with host buffers: problem creation
             (host -> device copies), the solve, and the read-back of T inside the timed region
   roofline  the dominant kernel: algorithmic bytes per launch / its mean CUDA-event duration,
@@ -359,6 +363,14 @@ def run_ours(args, rank, world, local_rank):
         torch.cuda.synchronize()
     barrier()
     ms = ev0.elapsed_time(ev1)
+    # the iterations after them as a caller's solve runs them (a first run captures its graphs)
+    plain_ms = []
+    for _ in range(2):
+        ev0.record(stream)
+        prob.solve(want_T=False, max_iters=args.steps, warm_start=1, **common)
+        ev1.record(stream)
+        torch.cuda.synchronize()
+        plain_ms.append(ev0.elapsed_time(ev1))
     from paper_2501_17996_gb300.sharding import aggregate_rate
 
     value, t_max = aggregate_rate(args.steps, ms / 1e3, world, device="cuda")
@@ -453,6 +465,7 @@ def run_ours(args, rank, world, local_rank):
                 "note": ("problem creation + upload, %d iterations, T read-back (after the device-resident "
                          "leg in the same process, so the device memory pool is warm)" % args.steps)},
         "gpu_launches": launches,
+        "solve": {"value": args.steps / (plain_ms[1] / 1e3), "ms_per_step": plain_ms[1] / args.steps},
         "clocks": clk.summary(),
         "cold_start": cold,
     }

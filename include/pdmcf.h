@@ -103,10 +103,10 @@ typedef struct mcf_options {
                                 iteration (rows of up to 1024 entries) or the flat node
                                 phase, and so does the index of the shape that it stands for
                                 (mcf_kernel_times.shape of a timed solve with -1); any other
-                                shape runs one launch per phase. (Many host threads that
-                                solve a network of 200 to 1024 nodes each: resident
-                                iterations take turns on the GPU, per-phase launches
-                                overlap, and mcf_solve_batch is the fastest of the three) */
+                                shape runs one launch per phase. (For four and more
+                                host threads that solve a network of 200 to 1024 nodes
+                                each: resident iterations take turns on the GPU, per-phase
+                                launches overlap, as does one mcf_solve_batch of them all) */
   double  adapt_guard;       /* g: stop adapting omega (keep it constant, Sec. 2.4) from
                                 the iteration after a stop test where omega is more than a
                                 factor g^2 away from its value at the first stop test with

@@ -226,8 +226,10 @@ project_row_kernel(ProjArgs a) {
 // group of the solver's shapes per column (GB300, 3e8 entries or 1e6 columns, normal columns, a
 // guess far below the multiplier): n = 100 428 -> 225 us, n = 200 612 -> 483, n = 400 708 -> 600,
 // n = 1000 673 -> 493, n = 3000 734 -> 571, n = 10 000 1081 -> 565 (4.3 TB/s; the rest is the
-// passes' arithmetic). With four lanes per column a launch of a few columns takes 7.8 us
-// against 5.8, so few columns keep the solver's shapes: a group per column from the first.
+// passes' arithmetic). Below `few` columns a group per column from the first (a pass of some 12 us
+// with its launch and events): shapes / variant in us, n = 400: 4096 columns 13.8 / 15.1, 8192 18.4 / 18.9,
+// 16 384 20.5 / 20.8; n = 1000: 2048 13.8 / 15.0, 4096 17.7 / 18.1; n = 3000: 512 14.0 / 16.0, 1024
+// 17.1 / 18.5, 2048 20.5 / 20.8; up to 200 entries both take 11.5 to 14 us below 16 384 columns.
 using ProjKernel = void (*)(ProjArgs);
 struct ProjVariant {
   ProjKernel fn;
