@@ -218,13 +218,12 @@ void mcf_options_default(mcf_options* o);
  * MCF_ERR_NUMERIC, MCF_ERR_OOM, MCF_ERR_CUDA or MCF_ERR_INVALID. */
 int mcf_solve(mcf_problem* p, const mcf_options* opts, mcf_result* res);
 
-/* Solve `count` independent problems together on one GPU (FP32 iterates only): the edge phase
- * is one launch per group of launch shapes and the other phases one launch each for all
- * resident problems, every problem keeps
- * its own step sizes, iteration count and stop test on the device, and its reductions are
- * summed per edge and per piece of a node's column in a fixed order, so a problem's iterates are identical
- * whether it is solved alone or in any batch. opts applies to every problem (warm_start = 1
- * continues each problem's resident iterate). results[i] is filled as by mcf_solve for
+/* Solve `count` independent problems together on one GPU (FP32 iterates only): the edge phase is
+ * one launch per group of launch shapes and the other phases one launch each for all resident
+ * problems, every problem keeps its own step sizes, iteration count and stop test on the device,
+ * and its reductions are summed per edge and per piece of a node's column in a fixed order, so a
+ * problem's iterates are identical whether it is solved alone or in any batch. opts applies to
+ * every problem (warm_start = 1 continues each problem's resident iterate). results[i] is filled as by mcf_solve for
  * problems[i], including any output buffers it points to. The problems must be distinct
  * and not in use by other calls. Returns MCF_OK if every problem met its stop rule, else
  * the first other status (results are still filled). */
@@ -309,8 +308,8 @@ int mcf_solve_timed(mcf_problem* p, const mcf_options* opts, mcf_result* res,
  *          order (independent of the launch grid)
  *   stream cudaStream_t (NULL = legacy default stream), on the calling thread's current device
  * With dist2, m+1 doubles of device scratch come from the pool that also holds the problems'
- * states, in stream order. Synchronizes the stream before returning. Errors: MCF_ERR_INVALID (sizes, NULL or misaligned pointers), MCF_ERR_OOM,
- * MCF_ERR_CUDA. */
+ * states, in stream order. Synchronizes the stream before returning. Errors: MCF_ERR_INVALID
+ * (sizes, NULL or misaligned pointers), MCF_ERR_OOM, MCF_ERR_CUDA. */
 int mcf_project_capped_simplex(int32_t n, int32_t m, int32_t ld, const float* Qt,
                                const float* cap, float* Ft, float* mu, double* dist2,
                                void* stream);

@@ -3,9 +3,10 @@
 //
 // Per iteration: an edge launch over the instances of each non-empty group of shapes, one node
 // and (where some instance takes a stop test) one check launch over all instances, then one
-// scalar launch with a block per instance. Instance scalars live on the device (BatchScalars), so a chunk of iterations is captured once as a
-// CUDA graph and replayed whatever the mix; the host reads the scalar mirror once per chunk
-// to retire finished instances and admit new ones between chunks.
+// scalar launch with a block per instance. Instance scalars live on the device (BatchScalars), so
+// a chunk of iterations is captured once as a CUDA graph and replayed whatever the mix; the host
+// reads the scalar mirror once per chunk to retire finished instances and admit new ones between
+// chunks.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -309,7 +310,6 @@ int BatchEngine::add(mcf_problem* p, const mcf_options& o, void* tag, int* slot_
   BCK(cudaMemcpyAsync(d_insts_ + s, &h_insts_[s], sizeof(bi), cudaMemcpyHostToDevice, stream_));
   BCK(cudaMemcpyAsync(d_sc_ + s, &hs, sizeof(hs), cudaMemcpyHostToDevice, stream_));
   (void)warm;
-  lists_dirty_ = true;
   *slot_out = s;
   return MCF_OK;
 }
@@ -605,9 +605,9 @@ int batch_class_for(int device, int nchunks, bool autotune) {
 
 using namespace pdmcf;
 
-// Solve `count` independent problems together (FP32; one launch per phase and shape class
-// for all of them). results[i] receives problem i's scalars and, if its T/F/Y pointers are
-// set, its outputs. Returns MCF_OK when every problem met its stop rule.
+// Solve `count` independent problems together (FP32; an edge launch per group of shapes and one
+// launch of each other phase for all of them). results[i] receives problem i's scalars and, if
+// its T/F/Y pointers are set, its outputs. Returns MCF_OK when every problem met its stop rule.
 extern "C" int mcf_solve_batch(mcf_problem** probs, int count, const mcf_options* opts,
                                mcf_result* results) {
   if (count < 0 || (count > 0 && (!probs || !results))) {
