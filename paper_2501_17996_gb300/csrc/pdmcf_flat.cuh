@@ -11,7 +11,7 @@ namespace pdmcf {
 // column block by column block. A row of F is gathered by its head and by its tail; within a block
 // both reads fall into the same few megabytes of F, so the second hits L2 where a pass node by
 // node read it from HBM again, and a thread has one chunk of a column instead of all of them.
-// n = 3000, m = 24 000 (FP32, log): 130 us at 3.8 TB/s of HBM and 46 % of issue slots, two FP32
+// n = 3000, m = 24 000 (FP32, log): 130 us, with DRAM and issue slots at 44 % each, two FP32
 // entries per lane (node_kernel without in-sums: 138 us); n = 1000 FP64 with an exponent per
 // pair: 2.5 -> 1.2 ms per iteration, bound by the FP64 unit.
 template <typename P, typename S, int N>

@@ -73,7 +73,7 @@ __device__ __forceinline__ void st_tail(__nv_bfloat16* p, const float (&v)[N]) {
 // Counter barrier over the CTAs of a cooperative launch, split in arrive and wait. The waits
 // are bounded (2^21 polls, a second or two): a CTA that gives up records wait_timeout and
 // leaves, the others run out of polls the same way, the launches queued behind this one return
-// at once (resident_start), and the driver reports MCF_ERR_CUDA.
+// at once (resident_start), and the solve reports MCF_ERR_CUDA.
 struct GridBarrier {
   unsigned* arrived;
   DevScalars* sc;

@@ -610,11 +610,12 @@ template <> const void* flat_kernel<double, double>() { return (const void*)flat
 // Renumbered networks, where the node phase's rows are close in memory anyway: n = 1500 113 -> 111,
 // n = 2000 178 -> 184. With exponents other than 1/2 the flat phase's root search decides:
 // n = 3000 559 -> 426.
-// BF16-stored F takes this path only where it gives the bits of the kernels it stands for: the
-// register shapes (the in-sum kind adds a node's in-edges in another order) with log utility (the
-// power search rounds differently). One last-place difference in Y or in a multiplier flips
-// roundings of F to BF16, each 2^-8 of an entry, and the flips spread: n = 3001, power, 100
-// iterations, T was 2.7e-3 (norm) from the per-phase kernels' with it.
+// BF16-stored F (log, n = 1500 97.6 -> 76.9, n = 2000 145 -> 129, kNN n = 1500 126 -> 104) takes this
+// path only where it gives the bits of the kernels it stands for: the register shapes (the in-sum
+// kind adds a node's in-edges in another order) with log utility (the power search rounds
+// differently). One last-place difference in Y or in a multiplier flips roundings of F to BF16, each
+// 2^-8 of an entry, and the flips spread: n = 3001, power, 100 iterations, T was 2.7e-3 (norm) from
+// the per-phase kernels' with it.
 template <typename P, typename S>
 static int setup_flat(DeviceState* d, int want) {
   d->grid_flat = 0;
