@@ -71,9 +71,10 @@ __device__ __forceinline__ void st_tail(__nv_bfloat16* p, const float (&v)[N]) {
 
 // ------------------------------------------------------------------ grid barrier
 // Counter barrier over the CTAs of a cooperative launch, split in arrive and wait. The waits
-// are bounded (2^21 polls, a second or two): a CTA that gives up records wait_timeout and
-// leaves, the others run out of polls the same way, the launches queued behind this one return
-// at once (resident_start), and the solve reports MCF_ERR_CUDA.
+// are bounded (2^22 polls, one to three seconds; a phase of the largest network that comes here,
+// 1024 nodes with every edge, takes well under a tenth of one): a CTA that gives up records
+// wait_timeout and leaves, the others run out of polls the same way, the launches queued behind
+// this one return at once (resident_start), and the solve reports MCF_ERR_CUDA.
 struct GridBarrier {
   unsigned* arrived;
   DevScalars* sc;
@@ -89,7 +90,7 @@ struct GridBarrier {
     if (threadIdx.x == 0) {
       unsigned v = 0;
       bool ok = false;
-      for (int it = 0; it < (1 << 21) && !ok; ++it) {
+      for (int it = 0; it < (1 << 22) && !ok; ++it) {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
         ok = (int)(v - target) >= 0;
       }

@@ -33,6 +33,7 @@ WORK = [
     (lambda: _powij(90, 6), dict(FIXED, precision="fp64", max_iters=300)),
     (lambda: I.ring_random_instance(260, 6, 7, "lognormal", "pow", gamma=0.4), FIXED),
     (lambda: _log(40, 4, 8), dict(FIXED, k_check=1)),
+    (lambda: _log(110, 8, 9), dict(FIXED, precision="bf16")),
 ]
 
 
