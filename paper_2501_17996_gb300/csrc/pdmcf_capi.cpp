@@ -410,6 +410,7 @@ int mcf_autotune(mcf_problem* p, const mcf_options* opts, int* best_shape, doubl
     mcf_options o = *opts;
     o.shape = s;
     o.stop_mode = MCF_STOP_NONE;
+    o.polish_iters = 0;   // the polish would replace the BF16 state after every run
     o.warm_start = 0;
     o.max_iters = 3;
     mcf_result r{};

@@ -48,3 +48,12 @@ def test_the_automatic_choice_by_its_name(lib, n, precision):
         a = p.solve(want_T=True, **opts)
         b = p.solve(want_T=True, shape=r["shape"], **opts)
     assert np.array_equal(a["T"], b["T"]) and a["omega"] == b["omega"]
+
+
+def test_tuning_bf16_storage_leaves_the_polish_out(lib):
+    """The FP32 polish after a BF16 phase has its own state and kernels: with it in every timed run
+    the time per iteration was that of an allocation and of polish_iters more iterations."""
+    with lib.Problem(I.ring_random_instance(600, 6, 4, "u1_10", "log")) as p:
+        _, plain = p.autotune(precision="bf16", stop_mode="none")
+        _, polished = p.autotune(precision="bf16", stop_mode="none", polish_iters=500)
+    assert polished <= 1.5 * plain
