@@ -389,7 +389,7 @@ int mcf_test_withhold_next_copy(void);
 /* Exercise the bounded waits of the resident iteration's grid barrier: the next solve on the
  * calling process that runs the resident iteration (automatic shape, rows of up to 1024
  * entries) waits at its first barrier for one arrival more than there are CTAs. Every CTA gives
- * up after 2^22 polls (one to three seconds) and leaves, the launches queued behind return at once,
+ * up after 2^22 polls (about a second) and leaves, the launches queued behind return at once,
  * and the solve ends with MCF_ERR_CUDA ("a bounded device-side wait timed out"). The problem's
  * iterate is then invalid, so the next solve starts cold. The paper has no counterpart. Returns
  * MCF_OK. */

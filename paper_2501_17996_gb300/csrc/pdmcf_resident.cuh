@@ -71,8 +71,8 @@ __device__ __forceinline__ void st_tail(__nv_bfloat16* p, const float (&v)[N]) {
 
 // ------------------------------------------------------------------ grid barrier
 // Counter barrier over the CTAs of a cooperative launch, split in arrive and wait. The waits
-// are bounded (2^22 polls, one to three seconds; a phase of the largest network that comes here,
-// 1024 nodes with every edge, takes well under a tenth of one): a CTA that gives up records
+// are bounded (2^22 polls, 0.9 s; an iteration of the largest network that comes here, 1024 nodes
+// with every edge, takes 5 ms in FP32 and 65 ms in FP64): a CTA that gives up records
 // wait_timeout and leaves, the others run out of polls the same way, the launches queued behind
 // this one return at once (resident_start), and the solve reports MCF_ERR_CUDA.
 struct GridBarrier {
